@@ -12,12 +12,22 @@
 //   UpdateCache: demand-loaded experts fill free slots, then each further one
 //   evicts the lowest-s^T resident outside S (the demand set's order does not
 //   change the resulting set, since inserted experts are in S and protected).
-// Reductions: the fp32 bit patterns of the (non-negative) scores serve as
-// ordered 32-bit keys.  Each lane keeps its keys sorted in policy order, so a
-// warp-wide "first in order" is one redux.sync (max key) and a ballot whose
-// lowest set lane owns it; a "last member" is a lane-local scan, a
-// redux.sync (min key) and a ballot whose highest set lane owns it.  Only the
-// owner lane learns which of its experts was picked.
+// Reductions: the fp32 bit patterns of the (non-negative) scores are ordered
+// like the scores, so a warp-wide extreme is a lane-local extreme and one
+// redux.sync; the slot that holds it finds itself by comparing, and a count of
+// the holders proves that there was exactly one.  Two holders (equal scores),
+// and a cache that is still filling, go to the general forms, which settle
+// every case by expert index with ballots.
+//
+// What bounds the step: the integer pipe (16 lanes a scheduler) when many
+// chains share an SM, and for a few chains the latency of some 300 dependent
+// instructions, a max/min redux.sync taking 23 cycles, an add 48.  Against the
+// step with integer masks, selects and one reduction after another: Qwen3
+// shape, stand-alone scan of 64 streams x 1000 tokens, 1.62 -> 1.27 ms for the
+// method, 1.06 -> 0.85 LRU, 1.24 -> 0.91 LFU, 1.39 -> 1.31 LRFU, 1.57 -> 1.39
+// Spatio-only; GPT-OSS shape (one expert a lane) 0.64 -> 0.44 ms, 0.34 -> 0.32,
+// 0.36 -> 0.33, 0.43 -> 0.43, 0.63 -> 0.52; one stream through the fused
+// kernel, 0.82 -> 0.65 us a token.
 #pragma once
 
 #include "crc_device.cuh"
@@ -69,6 +79,11 @@ __device__ __forceinline__ void presort(KeyList<V>& L) {
     }
 }
 
+template <int V>
+struct Keys {
+    uint32_t k[V];
+};
+
 // Removes the warp-wide first entry in policy order: the largest head key and,
 // among lanes whose head has it, the lowest lane (lanes own ascending index
 // ranges; a lane's head is its lowest index among equal keys).  Returns the
@@ -91,6 +106,27 @@ __device__ __forceinline__ int warp_pop_first(KeyList<V>& L, int lane, uint32_t&
         L.k[V - 1] = 0u;
     }
     return owner;
+}
+
+// The Top-K set of a row held by the warp (V keys a lane, 0 in invalid slots),
+// as V bits a lane, equal keys by ascending index: K pops with one owner each.
+template <int V>
+__device__ __noinline__ uint32_t topk_ties(Keys<V> key, uint32_t valid, int lane, int K) {
+    KeyList<V> P;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        P.k[v] = ((valid >> v) & 1u) ? key.k[v] + 1u : 0u;
+        P.s[v] = v;
+    }
+    presort<V>(P);
+    uint32_t sel = 0u;
+#pragma unroll 1
+    for (int k = 0; k < K; ++k) {
+        uint32_t kk, slot = 0u;
+        const int owner = warp_pop_first<V>(P, lane, kk, slot);
+        if (lane == owner) sel |= 1u << slot;
+    }
+    return sel;
 }
 
 // Last member in policy order among the slots flagged in `members`: smallest
@@ -123,6 +159,55 @@ struct Vec {
     float v[V];
 };
 
+// The stand-alone scans' rows pass through a ring in shared memory, filled
+// with cp.async scan_ahead tokens ahead of use: a step takes less than a trip to
+// L2 (480 cycles), let alone to DRAM, and a load into registers one step ahead
+// is waited for at the step's end (N = 32, 40 streams x 600 tokens: 0.79 us a
+// token for a chain's 144 instructions; 0.45 with the ring).  Every lane copies
+// and reads its own V floats, so no barrier is needed.
+template <int V>
+constexpr int scan_ahead() { return V >= 4 ? 4 : 8; }
+
+template <int V>
+__device__ __forceinline__ void ring_copy(float* dst, const float* src) {
+    const uint32_t at = smem_u32(dst);
+    if constexpr (V == 8) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at), "l"(src) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at + 16u), "l"(src + 4)
+                     : "memory");
+    } else if constexpr (V == 4) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at), "l"(src) : "memory");
+    } else if constexpr (V == 2) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(at), "l"(src) : "memory");
+    } else {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(at), "l"(src) : "memory");
+    }
+}
+__device__ __forceinline__ void ring_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void ring_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
+template <int V>
+__device__ __forceinline__ void ring_read(const float* src, float (&x)[V]) {
+    if constexpr (V >= 4) {
+#pragma unroll
+        for (int i = 0; i < V; i += 4) {
+            const float4 f = *reinterpret_cast<const float4*>(src + i);
+            x[i] = f.x;
+            x[i + 1] = f.y;
+            x[i + 2] = f.z;
+            x[i + 3] = f.w;
+        }
+    } else if constexpr (V == 2) {
+        const float2 f = *reinterpret_cast<const float2*>(src);
+        x[0] = f.x;
+        x[1] = f.y;
+    } else {
+        x[0] = *src;
+    }
+}
+
 template <int V>
 __device__ __forceinline__ Vec<V> load_vec(const float* p, bool ok) {
     Vec<V> r;
@@ -148,13 +233,102 @@ __device__ __forceinline__ Vec<V> load_vec(const float* p, bool ok) {
     return r;
 }
 
+// ---------------------------------------------------------------------------
+// The chain's step in fp32 arithmetic.  Residency is a 0 / 1 float per slot,
+// so masking a score, counting and updating the cache are FMA-pipe operations;
+// the integer pipe, whose 16 lanes a scheduler bound the scans when masks,
+// counts and updates were selects and integer adds (5 warps x 365 instructions
+// x 2 cycles a token for the Qwen3 shape), keeps the comparisons.
+// ---------------------------------------------------------------------------
+constexpr float kFar = 8.507059173023462e37f;   // 2^126; rows above it take the general forms
+
+// 1.0 where the comparison holds, else 0.0
+__device__ __forceinline__ float set_gt(float a, float b) {
+    float r;
+    asm("set.gt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float set_ge(float a, float b) {
+    float r;
+    asm("set.ge.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float set_eq(float a, float b) {
+    float r;
+    asm("set.eq.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+// Largest / smallest over the warp of non-negative floats, on their bits (whose
+// order is theirs; the compiler knows these reductions to be warp-uniform).
+__device__ __forceinline__ float warp_max_f(float x) {
+    return __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(x)));
+}
+__device__ __forceinline__ float warp_min_f(float x) {
+    return __uint_as_float(__reduce_min_sync(kFull, __float_as_uint(x)));
+}
+template <int V>
+__device__ __forceinline__ float lane_min_f(const float (&x)[V]) {
+    float r = x[0];
+#pragma unroll
+    for (int v = 1; v < V; ++v) r = fminf(r, x[v]);
+    return r;
+}
+template <int V>
+__device__ __forceinline__ float lane_max_f(const float (&x)[V]) {
+    float r = x[0];
+#pragma unroll
+    for (int v = 1; v < V; ++v) r = fmaxf(r, x[v]);
+    return r;
+}
+// Warp sum of lane values 2^23 + i, i a small whole number: the sum of the i.
+constexpr float kCount0 = 8388608.f;
+__device__ __forceinline__ uint32_t warp_count(float c) {
+    return __reduce_add_sync(kFull, __float_as_uint(c)) - 0x60000000u;   // 32 * bits(2^23)
+}
+
 // Chain-local state held in registers across tokens.
 template <int V>
 struct ChainRegs {
-    uint32_t cache;      // V bits: residency of this lane's experts
+    float out[V];        // 0 where this lane's expert is resident, else 1
     int count;           // |C| (warp-uniform)
     float aT[V];         // s^T of the previous token
     uint32_t hits, misses, pro;
+
+    __device__ __forceinline__ uint32_t bits(int) const {    // the residency as V bits
+        uint32_t b = 0u;
+#pragma unroll
+        for (int v = 0; v < V; ++v) b |= out[v] == 0.f ? 1u << v : 0u;
+        return b;
+    }
+    __device__ __forceinline__ void set_bits(uint32_t b) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) out[v] = ((b >> v) & 1u) ? 0.f : 1.f;
+    }
+};
+
+// Up to 32 experts, one a lane: the cache is one word, the same in every lane.
+template <>
+struct ChainRegs<1> {
+    uint32_t cache;
+    int count;
+    float aT[1];
+    uint32_t hits, misses, pro;
+
+    __device__ __forceinline__ uint32_t bits(int lane) const { return (cache >> lane) & 1u; }
+    __device__ __forceinline__ void set_bits(uint32_t b) {
+        cache = __ballot_sync(kFull, b & 1u);
+    }
+};
+
+// The native Top-K of an access: 0 / 1 per slot, or for one expert a lane the
+// set as one word.
+template <int V>
+struct Sel {
+    float s[V];
+};
+template <>
+struct Sel<1> {
+    uint32_t m;
 };
 
 // ---------------------------------------------------------------------------
@@ -298,10 +472,11 @@ __device__ __forceinline__ uint32_t take4(float4 f, float th, int& need) {
     return w;
 }
 
-// Top-K set of row[0..N) (N % 16 == 0, 1 <= K <= min(N, 32), values >= 0) as
-// bits mask[e / 32] bit e % 32; mask must hold N / 32 rounded up words.
+// K-th largest of row[0..N) (N % 16 == 0, 1 <= K <= min(N, 32), values >= 0):
+// the threshold of its Top-K set, which is every score at or above it unless
+// more than K are.
 template <int KP>
-__device__ __forceinline__ void row_topk_mask(const float* row, int N, int K, uint32_t* mask) {
+__device__ __forceinline__ float row_theta_k(const float* row, int N, int K) {
     TopKAcc<KP> acc;
     acc.init();
     for (int c = 0; c < N; c += 16) {
@@ -316,34 +491,7 @@ __device__ __forceinline__ void row_topk_mask(const float* row, int N, int K, ui
         }
         acc.add16(x);
     }
-    const float th = acc.theta(K);
-    // Every score >= theta: the Top-K set exactly when no more scores equal
-    // theta than the set takes (the usual case), i.e. when it has K members.
-    int cnt = 0;
-    for (int c = 0; c < N; c += 32) {
-        uint32_t w = 0u;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            if (c + 4 * q >= N) break;
-            const float4 f = __ldg(reinterpret_cast<const float4*>(row + c) + q);
-            w |= ((f.x >= th ? 1u : 0u) | (f.y >= th ? 2u : 0u) | (f.z >= th ? 4u : 0u) |
-                  (f.w >= th ? 8u : 0u)) << (4 * q);
-        }
-        mask[c >> 5] = w;
-        cnt += __popc(w);
-    }
-    if (cnt == K) return;
-    // surplus scores equal to theta: take the lowest indices among them
-    int need = acc.need(K, th);
-    for (int c = 0; c < N; c += 32) {
-        uint32_t w = 0u;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            if (c + 4 * q >= N) break;
-            w |= take4(__ldg(reinterpret_cast<const float4*>(row + c) + q), th, need) << (4 * q);
-        }
-        mask[c >> 5] = w;
-    }
+    return acc.theta(K);
 }
 
 // Algorithm 2's pre-access refinement of the chain's cache with priorities
@@ -362,21 +510,17 @@ __device__ __forceinline__ void row_topk_mask(const float* row, int N, int K, ui
 // the strict test, ending the pass exactly as the rank test or the strict
 // test ends it here.
 //
-// With nD_out, the first rank count also carries this lane's demand misses of
-// `sel` against the cache as it stands; when that count ends the pass (the
-// cache unchanged), *nD_out receives the warp's demand misses, else -1.
-template <int V, bool ALL_VALID>
-__device__ __forceinline__ int scan_refine(ChainRegs<V>& cr, const float (&pS)[V], uint32_t valid,
-                                           int lane, int C, int R, uint32_t sel = 0u,
-                                           int* nD_out = nullptr) {
-    auto is_valid = [&](int v) { return ALL_VALID || ((valid >> v) & 1u); };
-    uint32_t kS[V];
+// The general form, for a cache that is filling and for ties (keys: score bits,
+// 0 in invalid slots).  A function of its own, so the scans' loops stay short.
+// Returns the cache (V bits) | its count << 8 | the proactive loads << 20.
+template <int V>
+__device__ __noinline__ uint32_t refine_general(Keys<V> key, uint32_t cache, int count,
+                                                uint32_t valid, int lane, int C, int R) {
+    uint32_t kS[V];                            // the keys + 1, 0 in invalid slots
 #pragma unroll
-    for (int v = 0; v < V; ++v)
-        kS[v] = is_valid(v) ? pkey(__fadd_rn(cr.aT[v], pS[v])) : 0u;
-    uint32_t left = valid & ~cr.cache;         // non-residents not yet taken
+    for (int v = 0; v < V; ++v) kS[v] = ((valid >> v) & 1u) ? key.k[v] + 1u : 0u;
+    uint32_t left = valid & ~cache;            // non-residents not yet taken
     int pro = 0;
-    if (nD_out) *nD_out = -1;
 #pragma unroll 1
     for (int j = 0; j < R; ++j) {
         // the best remaining non-resident c: largest key, then lowest index
@@ -388,97 +532,296 @@ __device__ __forceinline__ int scan_refine(ChainRegs<V>& cr, const float (&pS)[V
         for (int v = 1; v < V; ++v) best = umax(best, m[v]);
         const uint32_t mx = __reduce_max_sync(kFull, best);
         if (mx == 0u) break;                   // no non-resident left
-        // rank of c: experts with higher keys, and with equal keys at lower
-        // indices (lanes before the owner; the owner's slots before c's).
-        // Invalid slots hold key 0 and count for neither.  Fields of 9 bits
-        // (counts <= N <= 256), the demand misses above them.
-        uint32_t gt = 0u, eq = 0u;
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            gt += kS[v] > mx ? 1u : 0u;
-            eq += kS[v] == mx ? 1u : 0u;
-        }
-        uint32_t packed = gt | (eq << 9);
-        if (nD_out && j == 0) packed |= (uint32_t)__popc(sel & ~cr.cache) << 18;
-        const uint32_t tot = __reduce_add_sync(kFull, packed);
-        uint32_t rank = tot & 0x1ffu;
-        const bool tie = ((tot >> 9) & 0x1ffu) > 1u;   // c shares its key
-        int owner = 0;
+        const int owner = __ffs(__ballot_sync(kFull, best == mx)) - 1;
         uint32_t cs = 0u;
-        auto locate = [&]() {                  // c's lane and slot
-            owner = __ffs(__ballot_sync(kFull, best == mx)) - 1;
 #pragma unroll
-            for (int v = V - 1; v >= 0; --v) cs = m[v] == mx ? (uint32_t)v : cs;   // lowest slot
-        };
-        if (tie) {                             // count those before c by index
-            locate();
-            const uint32_t c_slot = __shfl_sync(kFull, cs, owner);
-            uint32_t before = 0u;
+        for (int v = V - 1; v >= 0; --v) cs = m[v] == mx ? (uint32_t)v : cs;   // lowest slot
+        const uint32_t c_slot = __shfl_sync(kFull, cs, owner);
+        // rank of c: experts with higher keys, and with equal keys at lower indices
+        uint32_t before = 0u;
 #pragma unroll
-            for (int v = 0; v < V; ++v)
-                before += (kS[v] == mx && (lane < owner || (lane == owner && (uint32_t)v < c_slot)))
-                              ? 1u : 0u;
-            rank += __reduce_add_sync(kFull, before);
-        }
-        if ((int)rank >= R) {                  // c is not among the top R, nor is any later one
-            if (nD_out && j == 0) *nD_out = (int)(tot >> 18);
-            break;
-        }
-        if (!tie) locate();
+        for (int v = 0; v < V; ++v)
+            before += (kS[v] > mx ||
+                       (kS[v] == mx && (lane < owner || (lane == owner && (uint32_t)v < c_slot))))
+                          ? 1u : 0u;
+        if ((int)__reduce_add_sync(kFull, before) >= R) break;   // nor is any later one in A
         const uint32_t cbit = (lane == owner) ? (1u << cs) : 0u;
         left &= ~cbit;
-        if (cr.count < C) {                    // free slot: proactive load
-            cr.cache |= cbit;
-            ++cr.count;
+        if (count < C) {                       // free slot: proactive load
+            cache |= cbit;
+            ++count;
             ++pro;
             continue;
         }
         uint32_t kv, vslot = 0u;
-        const int vo = warp_last_member<V>(kS, cr.cache, lane, kv, vslot);
-        if (mx > kv) {                         // strictly higher: replace the lowest resident
-            const uint32_t vbit = (lane == vo) ? (1u << vslot) : 0u;
-            cr.cache = (cr.cache & ~vbit) | cbit;
+        const int vo = warp_last_member<V>(kS, cache, lane, kv, vslot);
+        if (mx <= kv) break;                   // later candidates are no higher
+        const uint32_t vbit = (lane == vo) ? (1u << vslot) : 0u;
+        cache = (cache & ~vbit) | cbit;        // strictly higher: replace the lowest resident
+        ++pro;
+    }
+    return cache | ((uint32_t)count << 8) | ((uint32_t)pro << 20);
+}
+
+// This lane's share of two counts over the warp: the demand misses of the
+// slots s (at most K <= 32) and, times 64, the members of s.
+template <int V>
+__device__ __forceinline__ float miss_count(const ChainRegs<V>& cr, const Sel<V>& sel) {
+    float miss = 0.f, all = 0.f;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        miss = __fmaf_rn(sel.s[v], cr.out[v], miss);
+        all = __fadd_rn(all, sel.s[v]);
+    }
+    return __fmaf_rn(all, 64.f, miss);
+}
+
+// The refinement with a full cache (every access but the first few): a round
+// takes the best non-resident's score and the lowest resident's in two
+// independent reductions, then one count that carries both c's rank and the
+// demand misses of the native Top-K s against the cache as it stands, so the
+// round that ends the pass has also counted them.  A swap is made by the
+// slots that hold the two scores, after a count has shown that each has one
+// holder, c's among all experts and the lowest's among the residents;
+// otherwise refine_general takes the pass on from the cache as it is.
+// *counts receives the demand misses and, above bit 6, the members of s.
+template <int V, bool ALL_VALID>
+__device__ __forceinline__ int scan_refine(ChainRegs<V>& cr, const float (&pS)[V], uint32_t valid,
+                                           int lane, int C, int R, const Sel<V>& s,
+                                           uint32_t* counts) {
+    float k[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        k[v] = __fadd_rn(cr.aT[v], pS[v]);
+        if (!ALL_VALID && !((valid >> v) & 1u)) k[v] = 0.f;
+    }
+    int pro = 0;
+    bool general = cr.count < C;
+    if (!general) {
+#pragma unroll 1
+        while (true) {
+            float x[V], y[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                x[v] = __fmul_rn(k[v], cr.out[v]);                 // invalid slots: 0
+                y[v] = __fmaf_rn(cr.out[v], kFar, k[v]);
+            }
+            const float mx = warp_max_f(lane_max_f<V>(x));
+            const float mn = warp_min_f(lane_min_f<V>(y));
+            float gt = kCount0;
+#pragma unroll
+            for (int v = 0; v < V; ++v) gt = __fadd_rn(gt, set_gt(k[v], mx));
+            const uint32_t tot = warp_count(__fmaf_rn(miss_count<V>(cr, s), 1024.f, gt));
+            *counts = tot >> 10;
+            // not among the top R, or no higher than the lowest resident: neither
+            // is any later candidate
+            if ((int)(tot & 1023u) >= R || __float_as_uint(mx) <= __float_as_uint(mn)) break;
+            float h = kCount0, in[V], go[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                in[v] = set_eq(k[v], mx);
+                go[v] = set_eq(y[v], mn);
+                h = __fadd_rn(h, in[v]);
+                h = __fmaf_rn(go[v], 1024.f, h);
+            }
+            general = warp_count(h) != 1025u || mn >= kFar;
+            if (general) break;
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                cr.out[v] = __fadd_rn(__fsub_rn(cr.out[v], in[v]), go[v]);
             ++pro;
-        } else {
-            break;                             // later candidates are no higher
         }
+    }
+    if (general) {
+        Keys<V> key;
+#pragma unroll
+        for (int v = 0; v < V; ++v) key.k[v] = __float_as_uint(k[v]);
+        const uint32_t r = refine_general<V>(key, cr.bits(lane), cr.count, valid, lane, C, R);
+        cr.set_bits(r & 0xffu);
+        cr.count = (int)((r >> 8) & 0xfffu);
+        pro += (int)(r >> 20);
+        *counts = warp_count(__fadd_rn(miss_count<V>(cr, s), kCount0));
     }
     return pro;
 }
 
+// The members (V bits) left after the n with the smallest keys, ties to the
+// highest index, are taken out one at a time.
+template <int V>
+__device__ __noinline__ uint32_t evict_general(Keys<V> key, uint32_t set, int n, int lane) {
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+        uint32_t kv, vslot = 0u;
+        const int vo = warp_last_member<V>(key.k, set, lane, kv, vslot);
+        if (lane == vo) set &= ~(1u << vslot);
+    }
+    return set;
+}
+
+// UpdateCache on a cache that overflows by n: of the residents outside S the n
+// with the smallest keys (ties to the highest index) leave, and S comes in;
+// `stay` of the former remain (their number is known: C - K).  Each round takes
+// every slot that holds the minimum; when a count then shows that equal keys
+// took more than n, the members are taken one at a time instead.  Ties are
+// rare among sums of probabilities (KeyTies::kRare); keys may also be known to
+// be distinct (kNone), or tie often (kOften: each round takes the highest
+// index among the holders of the minimum, one more reduction).
+enum class KeyTies { kNone, kRare, kOften };
+template <int V, KeyTies TIES>
+__device__ __forceinline__ void update_cache(ChainRegs<V>& cr, const float (&key)[V],
+                                             const Sel<V>& sel, int n, int stay, int lane) {
+    float y[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const float not_in = __fadd_rn(cr.out[v], __fmaf_rn(-cr.out[v], sel.s[v], sel.s[v]));
+        y[v] = __fmaf_rn(not_in, kFar, key[v]);
+    }
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+        const float mn = warp_min_f(lane_min_f<V>(y));
+        if constexpr (TIES == KeyTies::kOften) {
+            uint32_t at = 0u;                  // 1 + the highest index here that holds it
+#pragma unroll
+            for (int v = 0; v < V; ++v) at = y[v] == mn ? (uint32_t)(lane * V + v + 1) : at;
+            const uint32_t last = __reduce_max_sync(kFull, at);
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                y[v] = (uint32_t)(lane * V + v + 1) == last ? kFar : y[v];
+        } else {
+#pragma unroll
+            for (int v = 0; v < V; ++v) y[v] = __fmaf_rn(set_eq(y[v], mn), kFar, y[v]);
+        }
+    }
+    float gone[V], c = kCount0;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        gone[v] = set_ge(y[v], kFar);
+        c = __fadd_rn(c, gone[v]);
+    }
+    if (TIES == KeyTies::kRare && warp_count(c) != (uint32_t)(32 * V - stay)) {
+        Keys<V> all;
+        uint32_t set = 0u;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            all.k[v] = __float_as_uint(key[v]);
+            set |= (cr.out[v] == 0.f && sel.s[v] == 0.f) ? 1u << v : 0u;
+        }
+        set = evict_general<V>(all, set, n, lane);
+#pragma unroll
+        for (int v = 0; v < V; ++v) gone[v] = ((set >> v) & 1u) ? 0.f : 1.f;
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) cr.out[v] = __fmaf_rn(-sel.s[v], gone[v], gone[v]);
+}
+
+// The set of which a lane holds the V low bits of `bits`.
+template <int V>
+__device__ __forceinline__ void sel_from_bits(uint32_t bits, Sel<V>& sel) {
+    if constexpr (V == 1) {
+        sel.m = __ballot_sync(kFull, bits & 1u);
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) sel.s[v] = (bits & (1u << v)) ? 1.f : 0.f;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// One expert a lane (N <= 32): sets are words and counts are popcounts of
+// them, ties a choice of bit, so there is no general form to fall back to.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int refine_mask(ChainRegs<1>& cr, float pS, uint32_t valid, int lane,
+                                           int C, int R) {
+    const uint32_t bit = 1u << lane;
+    const uint32_t key = valid ? __float_as_uint(__fadd_rn(cr.aT[0], pS)) + 1u : 0u;
+    uint32_t left = __ballot_sync(kFull, valid != 0u) & ~cr.cache;   // not taken yet
+    int pro = 0;
+#pragma unroll 1
+    for (int j = 0; j < R; ++j) {
+        // the best remaining non-resident (ties: the lowest index), and the
+        // lowest resident (ties: the highest)
+        const uint32_t x = (left & bit) ? key : 0u;
+        const uint32_t y = (cr.cache & bit) ? key : 0xffffffffu;
+        const uint32_t mx = __reduce_max_sync(kFull, x);
+        const uint32_t mn = __reduce_min_sync(kFull, y);
+        const uint32_t c = __ballot_sync(kFull, x == mx) & left;
+        const uint32_t cbit = c & (0u - c);
+        const uint32_t ahead = __ballot_sync(kFull, key > mx) |
+                               (__ballot_sync(kFull, key == mx) & (cbit - 1u));
+        if (left == 0u || __popc(ahead) >= R) break;
+        left &= ~cbit;
+        if (cr.count < C) {
+            cr.cache |= cbit;
+            ++cr.count;
+        } else {
+            if (mx <= mn) break;
+            const uint32_t v = __ballot_sync(kFull, y == mn) & cr.cache;
+            cr.cache = (cr.cache & ~(0x80000000u >> __clz(v))) | cbit;
+        }
+        ++pro;
+    }
+    return pro;
+}
+
+// UpdateCache: of the residents outside `sel` the n with the smallest keys
+// leave (ties: the highest index), then `sel` is resident.
+__device__ __forceinline__ void update_mask(ChainRegs<1>& cr, uint32_t key, uint32_t sel, int n,
+                                            int lane) {
+    uint32_t w = cr.cache & ~sel;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+        const uint32_t y = ((w >> lane) & 1u) ? key : 0xffffffffu;
+        const uint32_t mn = __reduce_min_sync(kFull, y);
+        const uint32_t v = __ballot_sync(kFull, y == mn) & w;
+        w &= ~(0x80000000u >> __clz(v));
+    }
+    cr.cache = w | sel;
+}
+
 // Refinement, access and UpdateCache of one access, given s^T = p^R + p^T,
-// the Spatio prediction of the predecessor and the native Top-K set `sel`
-// (this lane's V bits).  Updates the chain registers; returns the number of
-// proactive loads and writes the demand misses to *n_miss.
-template <int V, bool ALL_VALID>
+// the Spatio prediction of the predecessor and the native Top-K as slots s (0
+// or 1), or as a word.  The counts show whether s has K members; if it has more (it was
+// taken by its threshold and scores tie there), exact_set(s) puts it right.
+// Updates the chain registers; returns the number of proactive loads and
+// writes the demand misses to *n_miss.  after_refine() is called between the
+// two phases.
+template <int V, bool ALL_VALID, class X, class F>
 __device__ __forceinline__ int scan_apply(ChainRegs<V>& cr, const float (&sT)[V],
                                           const float (&pS)[V], bool refine, uint32_t valid,
-                                          int lane, int K, int C, int R, uint32_t sel,
-                                          int* n_miss) {
-    int nD_pre = -1;
-    int pro = refine ? scan_refine<V, ALL_VALID>(cr, pS, valid, lane, C, R, sel, &nD_pre) : 0;
-
-    // demand misses and UpdateCache (Algorithm 1)
-    const uint32_t dem = sel & ~cr.cache;
-    const int nD = nD_pre >= 0 ? nD_pre : (int)__reduce_add_sync(kFull, (uint32_t)__popc(dem));
-    const int freeslots = C - cr.count;
-    if (nD > freeslots) {
-        uint32_t kT[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) kT[v] = pkey(sT[v]);
-        uint32_t vset = cr.cache & ~sel;                       // V = C+ \ S
-        for (int i = 0; i < nD - freeslots; ++i) {
-            uint32_t kv, vslot = 0u;
-            const int vo = warp_last_member<V>(kT, vset, lane, kv, vslot);
-            const uint32_t rm = (lane == vo) ? (1u << vslot) : 0u;
-            vset &= ~rm;
-            cr.cache &= ~rm;
-        }
-        cr.count = C;
+                                          int lane, int K, int C, int R, Sel<V>& s,
+                                          int* n_miss, X exact_set, F after_refine) {
+    int pro = 0, nD;
+    if constexpr (V == 1) {
+        if (refine) pro = refine_mask(cr, pS[0], valid, lane, C, R);
+        after_refine();
+        if (__popc(s.m) != K) exact_set(s);
+        nD = __popc(s.m & ~cr.cache);
+        const int over = cr.count + nD - C;
+        update_mask(cr, __float_as_uint(sT[0]), s.m, over, lane);
+        cr.count = over > 0 ? C : cr.count + nD;
     } else {
-        cr.count += nD;
+        uint32_t counts;
+        if (refine)
+            pro = scan_refine<V, ALL_VALID>(cr, pS, valid, lane, C, R, s, &counts);
+        else
+            counts = warp_count(__fadd_rn(miss_count<V>(cr, s), kCount0));
+        after_refine();
+        if ((counts >> 6) != (uint32_t)K) {
+            exact_set(s);
+            counts = warp_count(__fadd_rn(miss_count<V>(cr, s), kCount0));
+        }
+        nD = (int)(counts & 63u);
+
+        // demand misses and UpdateCache (Algorithm 1)
+        const int over = cr.count + nD - C;
+        if (over > 0) {
+            update_cache<V, KeyTies::kRare>(cr, sT, s, over, C - K, lane);
+            cr.count = C;
+        } else if (nD > 0) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) cr.out[v] = __fmaf_rn(-s.s[v], cr.out[v], cr.out[v]);
+            cr.count += nD;
+        }
     }
-    cr.cache |= dem;
 #pragma unroll
     for (int v = 0; v < V; ++v) cr.aT[v] = sT[v];
     cr.hits += (uint32_t)(K - nD);
@@ -488,74 +831,82 @@ __device__ __forceinline__ int scan_apply(ChainRegs<V>& cr, const float (&sT)[V]
     return pro;
 }
 
-// This lane's cache bits as the chain's NW bitmask words at dst.
+// The slots at or above the Top-K threshold of the row p.
+template <int V, bool ALL_VALID>
+__device__ __forceinline__ void sel_above(const float (&p)[V], float theta, uint32_t valid,
+                                          Sel<V>& sel) {
+    if constexpr (V == 1) {
+        sel.m = __ballot_sync(kFull, valid != 0u && p[0] >= theta);
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+            sel.s[v] = (ALL_VALID || ((valid >> v) & 1u)) ? set_ge(p[v], theta) : 0.f;
+    }
+}
+// The Top-K set of a row whose threshold ties.
 template <int V>
-__device__ __forceinline__ void store_cache_words(uint32_t cache, int lane, int N, uint32_t* dst) {
-    const int NW = (N + 31) >> 5;
-    const int e0 = lane * V;
-    for (int w = 0; w < NW; ++w) {
-        const uint32_t contrib = (e0 < N && (e0 >> 5) == w) ? (cache << (e0 & 31)) : 0u;
-        const uint32_t word = __reduce_or_sync(kFull, contrib);
-        if (lane == 0) dst[w] = word;
+__device__ __forceinline__ void sel_ties(const float (&p)[V], uint32_t valid, int lane, int K,
+                                         Sel<V>& sel) {
+    Keys<V> key;
+#pragma unroll
+    for (int v = 0; v < V; ++v) key.k[v] = __float_as_uint(p[v]);
+    sel_from_bits<V>(topk_ties<V>(key, valid, lane, K), sel);
+}
+// This lane's V bits of the set.
+template <int V>
+__device__ __forceinline__ uint32_t sel_bits(const Sel<V>& sel, int lane) {
+    if constexpr (V == 1) {
+        return (sel.m >> lane) & 1u;
+    } else {
+        uint32_t b = 0u;
+#pragma unroll
+        for (int v = 0; v < V; ++v) b |= sel.s[v] != 0.f ? 1u << v : 0u;
+        return b;
     }
 }
 
-// One access at (t, l) from the three router probabilities: s^T, the native
-// Top-K (given as a set, or popped in rank order when the trace wants the
-// order), then scan_apply.  Writes the trace.
-template <int V, bool ALL_VALID>
-__device__ __forceinline__ void scan_step(ChainRegs<V>& cr, const float (&pR)[V],
-                                          const float (&pT)[V], const float (&pS)[V],
-                                          bool refine, uint32_t valid, int lane, int K, int C,
-                                          int R, bool have_sel, uint32_t sel_in,
-                                          uint8_t* topk_out, uint8_t* miss_out,
-                                          uint8_t* pro_out, uint32_t* mid_out = nullptr,
-                                          uint32_t* after_out = nullptr, int N = 0,
-                                          uint32_t* sel_out = nullptr) {
-    auto is_valid = [&](int v) { return ALL_VALID || ((valid >> v) & 1u); };
-    float sT[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v) sT[v] = __fadd_rn(pR[v], pT[v]);
-
-    uint32_t sel = sel_in;
-    int my_topk = 0;
-    const bool want_topk = topk_out != nullptr;
-    if (!have_sel) {
-        KeyList<V> P;
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            P.k[v] = is_valid(v) ? pkey(pR[v]) : 0u;
-            P.s[v] = v;
-        }
-        presort<V>(P);
-        sel = 0u;
-        for (int k = 0; k < K; ++k) {
-            uint32_t kk, slot = 0u;
-            const int owner = warp_pop_first<V>(P, lane, kk, slot);
-            if (lane == owner) sel |= 1u << slot;
-            if (want_topk) {
-                const int e = __shfl_sync(kFull, lane * V + (int)slot, owner);
-                if (lane == k) my_topk = e;
-            }
-        }
-    }
-    int nD, pro;
-    if (mid_out) {
-        // the refinement on its own, so the cache between the two phases is seen
-        pro = refine ? scan_refine<V, ALL_VALID>(cr, pS, valid, lane, C, R) : 0;
-        store_cache_words<V>(cr.cache, lane, N, mid_out);
-        scan_apply<V, ALL_VALID>(cr, sT, pS, false, valid, lane, K, C, R, sel, &nD);
-        cr.pro += (uint32_t)pro;
+// This lane's V bits of a set as the set's NW bitmask words at dst (4-byte
+// aligned): the warp's bits are gathered to whole bytes (one ballot for V = 1;
+// log2(8 / V) shuffles otherwise) and stored bytewise, 4 NW bytes in one
+// store.  (One redux.or and one store a word took four of each for N = 128.)
+template <int V>
+__device__ __forceinline__ void store_cache_words(uint32_t bits, int lane, int N, uint32_t* dst) {
+    const int NW = (N + 31) >> 5;
+    if constexpr (V == 1) {
+        const uint32_t word = __ballot_sync(kFull, bits & 1u);
+        if (lane == 0) dst[0] = word;
     } else {
-        pro = scan_apply<V, ALL_VALID>(cr, sT, pS, refine, valid, lane, K, C, R, sel, &nD);
+#pragma unroll
+        for (int o = 1; o * V < 8; o <<= 1)
+            bits |= __shfl_down_sync(kFull, bits, o) << (o * V);
+        const int byte = lane * V / 8;
+        if (lane % (8 / V) == 0 && byte < 4 * NW)
+            reinterpret_cast<uint8_t*>(dst)[byte] = (uint8_t)bits;
     }
-    if (after_out) store_cache_words<V>(cr.cache, lane, N, after_out);
-    if (sel_out) store_cache_words<V>(sel, lane, N, sel_out);
-    if (want_topk && lane < K) topk_out[lane] = (uint8_t)my_topk;
-    if (lane == 0) {
-        if (miss_out) *miss_out = (uint8_t)nD;
-        if (pro_out) *pro_out = (uint8_t)pro;
+}
+
+// The native Top-K in rank order, for a trace that wants it: returns the set.
+template <int V>
+__device__ __forceinline__ uint32_t topk_ranked(const float (&pR)[V], uint32_t valid, int lane,
+                                                int K, uint8_t* topk_out) {
+    KeyList<V> P;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        P.k[v] = ((valid >> v) & 1u) ? pkey(pR[v]) : 0u;
+        P.s[v] = v;
     }
+    presort<V>(P);
+    uint32_t sel = 0u;
+    int mine = 0;
+    for (int k = 0; k < K; ++k) {
+        uint32_t kk, slot = 0u;
+        const int owner = warp_pop_first<V>(P, lane, kk, slot);
+        if (lane == owner) sel |= 1u << slot;
+        const int e = __shfl_sync(kFull, lane * V + (int)slot, owner);
+        if (lane == k) mine = e;
+    }
+    if (lane < K) topk_out[lane] = (uint8_t)mine;
+    return sel;
 }
 
 // Bits of this lane's experts from the chain's bitmask words.
@@ -578,8 +929,6 @@ constexpr int kScanWarps = 1;
 template <int V, bool ALL_VALID, int KP, bool TRACED>
 __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWarps)
     cache_scan_kernel(ScanArgs a) {
-    // Top-K sets of the next 32 tokens of each warp's chain, one row per token
-    __shared__ uint32_t sel_s[kScanWarps][32][8];
     StateHeader* hdr = reinterpret_cast<StateHeader*>(a.state);
     const StateLayout lay = state_layout(a.B, a.L, a.N);
     ChainState* chains = reinterpret_cast<ChainState*>(a.state + lay.chains);
@@ -610,8 +959,9 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
 
         ChainState& cs = chains[chain];
         ChainRegs<V> cr;
-        cr.cache = lane_bits<V>(cs.bits, lane, N);
-        cr.count = (int)__reduce_add_sync(kFull, (uint32_t)__popc(cr.cache));
+        const uint32_t resident = lane_bits<V>(cs.bits, lane, N);
+        cr.set_bits(resident);
+        cr.count = (int)__reduce_add_sync(kFull, (uint32_t)__popc(resident));
         {
             Vec<V> x = load_vec<V>(retention + (size_t)chain * N + lane * V, has);
 #pragma unroll
@@ -619,97 +969,108 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
         }
         cr.hits = cr.misses = cr.pro = 0u;
 
-        const float* base = a.scores + lane * V;
         // debug builds: the unit a pointer is formed for lies inside scores [B][T][L]
         auto unit_ok = [&](int t, int ll) {
             return CRC_IN_BOUNDS(b < a.B && t >= 0 && t < T && ll >= 0 && ll < L, err);
         };
-        auto unit_ptr = [&](int t, int ll) -> const float* {
-            return base + (((size_t)b * T + t) * L + ll) * row;
-        };
-        const float* carry_in = carry + ((size_t)parity * a.B + b) * N + lane * V;
-        auto pred_ptr = [&](int t) -> const float* {     // p^S of rho(t, l)
-            if (l > 0) return unit_ptr(t, l - 1) + 2 * N;
-            if (t > 0) return unit_ptr(t - 1, L - 1) + 2 * N;
-            return carry_in;
-        };
-        const bool want_s = a.R > 0;
-
-        // Without a trace only the Top-K *set* is needed: it does not depend on
-        // the cache, so lane j computes it for token t + j ahead of the chain.
-        const bool batch_sel = !TRACED || a.trace_topk == nullptr;
-        uint32_t (*sel_rows)[8] = sel_s[(threadIdx.x >> 5) % kScanWarps];
-        const float* row_base = a.scores + ((size_t)b * T * L + l) * row;   // token 0 of chain
         // running pointer to this lane's part of unit (b, t, l); p^S of rho(t, l)
-        // sits at a fixed offset from it: unit (t, l-1), or (t-1, L-1) for l = 0
+        // sits at a fixed offset from it: unit (t, l-1), or (t-1, L-1) for l = 0,
+        // whose first token takes the carry
+        const float* row0 = a.scores + ((size_t)b * T * L + l) * row;       // token 0 of the chain
+        const float* carry_in = carry + ((size_t)parity * a.B + b) * N + lane * V;
         const size_t tok = (size_t)L * row;
         const ptrdiff_t s_off = l > 0 ? (ptrdiff_t)2 * N - (ptrdiff_t)row
                                       : (ptrdiff_t)(L - 1) * (ptrdiff_t)row - (ptrdiff_t)tok +
                                             (ptrdiff_t)2 * N;
-        const float* up = unit_ptr(0, l);
+        const bool want_s = a.R > 0;
+        const bool rank_order = TRACED && a.trace_topk != nullptr;
 
-        Vec<V> cR = load_vec<V>(unit_ptr(0, l), has && unit_ok(0, l));
-        Vec<V> cT = load_vec<V>(unit_ptr(0, l) + N, has && unit_ok(0, l));
-        Vec<V> cS = load_vec<V>(pred_ptr(0), has && want_s && (t0 + 0 >= 1) &&
-                                                 (l > 0 ? unit_ok(0, l - 1) : true));
-        for (int t = 0; t < T; ++t) {
-            if (batch_sel && (t & 31) == 0) {
-                __syncwarp();
-                if (t + lane < T && unit_ok(t + lane, l)) {
-                    const float* r = row_base + (size_t)(t + lane) * L * row;
-                    row_topk_mask<KP>(r, N, a.K, sel_rows[lane]);
-                }
-                __syncwarp();
-            }
-            uint32_t sel_in = 0u;
-            if (batch_sel && has) {
-                const uint32_t e0 = (uint32_t)lane * V;
-                if (CRC_IN_BOUNDS((e0 >> 5) < 8u, err))
-                    sel_in = (sel_rows[t & 31][e0 >> 5] >> (e0 & 31)) & ((1u << V) - 1u);
-            }
-            Vec<V> nR, nT, nS;
-            if (t + 1 < T) {
-                const bool ok1 = unit_ok(t + 1, l);
-                const float* un = up + tok;
-                nR = load_vec<V>(un, has && ok1);
-                nT = load_vec<V>(un + N, has && ok1);
-                nS = load_vec<V>(un + s_off, has && want_s &&
-                                                 (l > 0 ? unit_ok(t + 1, l - 1) : unit_ok(t, L - 1)));
-            }
-            up += tok;
-            const bool refine = want_s && (t0 + t >= 1);
-            if constexpr (TRACED) {
-                const size_t unit = ((size_t)b * a.trace_T + a.trace_t0 + t) * L + l;
-                const size_t NWs = (size_t)((N + 31) >> 5);
-                scan_step<V, ALL_VALID>(cr, cR.v, cT.v, cS.v, refine, valid, lane, a.K, a.C, a.R,
-                                        batch_sel, sel_in,
-                                        a.trace_topk ? a.trace_topk + unit * a.K : nullptr,
-                                        a.trace_miss ? a.trace_miss + unit : nullptr,
-                                        a.trace_pro ? a.trace_pro + unit : nullptr,
-                                        a.trace_mid ? a.trace_mid + unit * NWs : nullptr,
-                                        a.trace_after ? a.trace_after + unit * NWs : nullptr, N,
-                                        a.trace_sel ? a.trace_sel + unit * NWs : nullptr);
-            } else {                      // no trace: the set-valued Top-K, straight to the step
-                float sT[V];
+        constexpr int D = scan_ahead<V>();
+        __shared__ __align__(16) float ring[kScanWarps][D][3][32 * V];
+        float (*mine)[3][32 * V] = ring[(threadIdx.x >> 5) % kScanWarps];
+        if (!has) {                              // slots past N read as 0
 #pragma unroll
-                for (int v = 0; v < V; ++v) sT[v] = __fadd_rn(cR.v[v], cT.v[v]);
-                int nD;
-                scan_apply<V, ALL_VALID>(cr, sT, cS.v, refine, valid, lane, a.K, a.C, a.R, sel_in,
-                                         &nD);
+            for (int i = 0; i < D * 3; ++i)
+#pragma unroll
+                for (int v = 0; v < V; ++v) mine[i / 3][i % 3][lane * V + v] = 0.f;
+        }
+        const float* up = row0 + lane * V;
+        auto load = [&](int t) {                 // t: the token `up` points at
+            if (t < T && has && unit_ok(t, l)) {
+                float (*to)[32 * V] = mine[t % D];
+                const bool first = l == 0 && t == 0;
+                ring_copy<V>(&to[0][lane * V], up);
+                ring_copy<V>(&to[1][lane * V], up + N);
+                if (want_s && t0 + t >= 1 &&
+                    (first || unit_ok(l > 0 ? t : t - 1, l > 0 ? l - 1 : L - 1)))
+                    ring_copy<V>(&to[2][lane * V], first ? carry_in : up + s_off);
+            }
+            ring_commit();
+            up += tok;
+        };
+        // The Top-K thresholds do not depend on the cache: lane j takes that of
+        // token t + j for t a multiple of 32; th is the current token's.
+        float theta = 0.f, th = 0.f;
+        auto step = [&](int t) {
+            float pR[V], pT[V], pS[V];
+            float (*from)[32 * V] = mine[t % D];
+            ring_read<V>(&from[0][lane * V], pR);
+            ring_read<V>(&from[1][lane * V], pT);
+            ring_read<V>(&from[2][lane * V], pS);
+            if ((t & 31) == 0) {
+                if (t + lane < T && unit_ok(t + lane, l))
+                    theta = row_theta_k<KP>(row0 + (size_t)(t + lane) * tok, N, a.K);
+                th = __shfl_sync(kFull, theta, 0);
+            }
+            Sel<V> s;
+            float sT[V];
+            if (!rank_order) sel_above<V, ALL_VALID>(pR, th, valid, s);
+            const size_t unit = ((size_t)b * a.trace_T + a.trace_t0 + t) * L + l;
+            const size_t NWs = (size_t)((N + 31) >> 5);
+            if (rank_order)
+                sel_from_bits<V>(
+                    topk_ranked<V>(pR, valid, lane, a.K, a.trace_topk + unit * a.K), s);
+#pragma unroll
+            for (int v = 0; v < V; ++v) sT[v] = __fadd_rn(pR[v], pT[v]);
+            int nD;
+            const int pro = scan_apply<V, ALL_VALID>(
+                cr, sT, pS, want_s && t0 + t >= 1, valid, lane, a.K, a.C, a.R, s, &nD,
+                [&](Sel<V>& x) { sel_ties<V>(pR, valid, lane, a.K, x); },
+                [&] {
+                    if (TRACED && a.trace_mid)
+                        store_cache_words<V>(cr.bits(lane), lane, N, a.trace_mid + unit * NWs);
+                });
+            if constexpr (TRACED) {
+                if (a.trace_after)
+                    store_cache_words<V>(cr.bits(lane), lane, N, a.trace_after + unit * NWs);
+                if (a.trace_sel)
+                    store_cache_words<V>(sel_bits<V>(s, lane), lane, N, a.trace_sel + unit * NWs);
+                if (lane == 0) {
+                    if (a.trace_miss) a.trace_miss[unit] = (uint8_t)nD;
+                    if (a.trace_pro) a.trace_pro[unit] = (uint8_t)pro;
+                }
             }
             // debug builds: every expert the step made resident lies in this
             // lane's range and the cache holds at most C experts
-            (void)CRC_IN_BOUNDS((cr.cache & ~valid) == 0u && cr.count <= a.C, err);
-            cR = nR;
-            cT = nT;
-            cS = nS;
+            (void)CRC_IN_BOUNDS((cr.bits(lane) & ~valid) == 0u && cr.count <= a.C, err);
+        };
+#pragma unroll
+        for (int t = 0; t < D - 1; ++t) load(t);
+        // (One copy of the step in the loop: two, with registers in place of the
+        // ring, ran a lone chain 13 % slower for the longer code.)
+#pragma unroll 1
+        for (int t = 0; t < T; ++t) {
+            load(t + D - 1);
+            ring_wait<D - 1>();                  // token t's copies have landed
+            step(t);
+            th = __shfl_sync(kFull, theta, (t + 1) & 31);
         }
 
         // write back the chain
         const int NW = (N + 31) >> 5;
         for (int w = 0; w < NW; ++w) {
             const int e0 = lane * V;
-            const uint32_t contrib = (has && (e0 >> 5) == w) ? (cr.cache << (e0 & 31)) : 0u;
+            const uint32_t contrib = (has && (e0 >> 5) == w) ? (cr.bits(lane) << (e0 & 31)) : 0u;
             const uint32_t word = __reduce_or_sync(kFull, contrib);
             if (lane == 0) cs.bits[w] = word;
         }
@@ -725,7 +1086,7 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
         }
         // the last layer hands its final p^S to layer 0 of the next call
         if (l == L - 1 && has) {
-            const float* src = unit_ptr(T - 1, L - 1) + 2 * N;
+            const float* src = row0 + lane * V + (size_t)(T - 1) * tok + 2 * N;
             float* dst = carry + ((size_t)(parity ^ 1u) * a.B + b) * N + lane * V;
 #pragma unroll
             for (int v = 0; v < V; ++v)

@@ -234,8 +234,9 @@ __device__ __forceinline__ void fused_scan_role(const FusedArgs& a, uint32_t* er
 
         ChainState& cs = chains[chain];
         ChainRegs<V> cr;
-        cr.cache = lane_bits_cg<V>(cs.bits, lane, N);
-        cr.count = (int)__reduce_add_sync(kFull, (uint32_t)__popc(cr.cache));
+        const uint32_t resident = lane_bits_cg<V>(cs.bits, lane, N);
+        cr.set_bits(resident);
+        cr.count = (int)__reduce_add_sync(kFull, (uint32_t)__popc(resident));
         {
             Vec<V> x = ldcg_vec<V>(retention + (size_t)chain * N + e0, has);
 #pragma unroll
@@ -295,45 +296,44 @@ __device__ __forceinline__ void fused_scan_role(const FusedArgs& a, uint32_t* er
         };
         prefetch_rows(8);
         prefetch_rows(16);
-        float cT[V], cS[V];
-        uint32_t csel;
-        fetch(0, cT, cS, csel);
-        for (int tbi = 0; tbi < steps; ++tbi) {
-            float nT[V], nS[V];
-            uint32_t nsel = 0u;
-            if (tbi + 1 < steps) fetch(tbi + 1, nT, nS, nsel);
+        // a step's record is fetched one step ahead
+        struct In {
+            float T[V], S[V];
+            uint32_t selw;
+        };
+        auto step = [&](int tbi, const In& q) {
             if ((tbi & 7) == 0) prefetch_rows(tbi + 24);
-            const bool refine = want_s && tbi >= refine_from;
-            const uint32_t sel = (csel >> (e0 & 31)) & ((1u << V) - 1u);
+            Sel<V> s;
+            sel_from_bits<V>(q.selw >> (e0 & 31), s);
+            const bool tr = traced && CRC_IN_BOUNDS(tb * a.TB + tbi < a.T, err);
+            const size_t unit = ((size_t)b * a.T + tb * a.TB + tbi) * L + l;
             int nD;
-            if (traced && CRC_IN_BOUNDS(tb * a.TB + tbi < a.T, err)) {
-                // the refinement on its own, so the cache between the phases is seen
-                const size_t unit = ((size_t)b * a.T + tb * a.TB + tbi) * L + l;
-                const int pro = refine ? scan_refine<V, ALL_VALID>(cr, cS, valid, lane, a.C, a.R)
-                                       : 0;
-                if (a.tr_mid) store_cache_words<V>(cr.cache, lane, N, a.tr_mid + unit * NW);
-                scan_apply<V, ALL_VALID>(cr, cT, cS, false, valid, lane, a.K, a.C, a.R, sel,
-                                         &nD);
-                cr.pro += (uint32_t)pro;
-                if (a.tr_after) store_cache_words<V>(cr.cache, lane, N, a.tr_after + unit * NW);
-                if (a.tr_sel && has && (e0 & 31u) == 0u) a.tr_sel[unit * NW + (e0 >> 5)] = csel;
+            const int pro = scan_apply<V, ALL_VALID>(
+                cr, q.T, q.S, want_s && tbi >= refine_from, valid, lane, a.K, a.C, a.R, s, &nD,
+                [](Sel<V>&) {},
+                [&] {
+                    if (tr && a.tr_mid)
+                        store_cache_words<V>(cr.bits(lane), lane, N, a.tr_mid + unit * NW);
+                });
+            if (tr) {
+                if (a.tr_after) store_cache_words<V>(cr.bits(lane), lane, N, a.tr_after + unit * NW);
+                if (a.tr_sel && has && (e0 & 31u) == 0u) a.tr_sel[unit * NW + (e0 >> 5)] = q.selw;
                 if (lane == 0) {
                     if (a.tr_miss) a.tr_miss[unit] = (uint8_t)nD;
                     if (a.tr_pro) a.tr_pro[unit] = (uint8_t)pro;
                 }
-            } else {
-                scan_apply<V, ALL_VALID>(cr, cT, cS, refine, valid, lane, a.K, a.C, a.R, sel,
-                                         &nD);
             }
             // debug builds: every expert the step made resident lies in this
             // lane's range and the cache holds at most C experts
-            (void)CRC_IN_BOUNDS((cr.cache & ~valid) == 0u && cr.count <= a.C, err);
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                cT[v] = nT[v];
-                cS[v] = nS[v];
-            }
-            csel = nsel;
+            (void)CRC_IN_BOUNDS((cr.bits(lane) & ~valid) == 0u && cr.count <= a.C, err);
+        };
+        In q, next;
+        fetch(0, q.T, q.S, q.selw);
+#pragma unroll 1
+        for (int tbi = 0; tbi < steps; ++tbi) {
+            if (tbi + 1 < steps) fetch(tbi + 1, next.T, next.S, next.selw);
+            step(tbi, q);
+            q = next;
         }
         // the last layer hands p^S of the call's last token to layer 0 of the next call
         if (l == L - 1 && want_s && tb * a.TB + a.TB >= a.T && steps > 0 && has) {
@@ -346,7 +346,7 @@ __device__ __forceinline__ void fused_scan_role(const FusedArgs& a, uint32_t* er
         }
         // store the chain
         for (int w = 0; w < NW; ++w) {
-            const uint32_t contrib = (has && (e0 >> 5) == (uint32_t)w) ? (cr.cache << (e0 & 31)) : 0u;
+            const uint32_t contrib = (has && (e0 >> 5) == (uint32_t)w) ? (cr.bits(lane) << (e0 & 31)) : 0u;
             const uint32_t wd = __reduce_or_sync(kFull, contrib);
             if (lane == 0) cs.bits[w] = wd;
         }

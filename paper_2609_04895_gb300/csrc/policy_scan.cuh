@@ -44,78 +44,91 @@ __device__ __forceinline__ float lrfu_decay(int lambda2, uint32_t dt) {
 // own priority arithmetic).  aux: this lane's integer priorities (LRU,
 // Spatio-only, LRFU: token of last use; LFU: count); cr.aT: the float ones
 // (LRFU: CRF; Spatio-only: p^R of the previous token).
-template <int V, bool ALL_VALID, int POL>
+template <int V, bool ALL_VALID, int POL, class X>
 __device__ __forceinline__ void policy_step(ChainRegs<V>& cr, uint32_t (&aux)[V],
                                             const float (&pR)[V], const float (&pS)[V],
                                             bool refine, uint32_t valid, int lane,
-                                            const PolicyArgs& a, uint32_t t, bool have_sel,
-                                            uint32_t sel_in, uint8_t* topk_out,
-                                            uint8_t* miss_out, uint8_t* pro_out) {
-    auto is_valid = [&](int v) { return ALL_VALID || ((valid >> v) & 1u); };
+                                            const PolicyArgs& a, uint32_t t, Sel<V>& s,
+                                            X exact_set, uint8_t* miss_out, uint8_t* pro_out) {
     const int K = a.s.K, C = a.s.C;
-    int pro = 0;
-    if (POL == CRC_POLICY_SPATIO_LRU && refine) {
-        const uint32_t before = cr.cache;
-        pro = scan_refine<V, ALL_VALID>(cr, pS, valid, lane, C, a.s.R);
-        const uint32_t loaded = cr.cache & ~before;
+    int pro = 0, nD;
+    bool in_s[V], was_in[V];                   // S, and the cache before the demand loads
+    // the priority that evicts, as an ordered word
+    auto word = [&](int v) {
+        return POL == CRC_POLICY_LRFU ? __float_as_uint(__fmul_rn(
+                                            cr.aT[v], lrfu_decay(a.lambda2, t - aux[v])))
+                                      : aux[v];
+    };
+    if constexpr (V == 1) {
+        if (POL == CRC_POLICY_SPATIO_LRU && refine) {
+            const uint32_t before = cr.cache;
+            pro = refine_mask(cr, pS[0], valid, lane, C, a.s.R);
+            if (((cr.cache & ~before) >> lane) & 1u) aux[0] = t;
+        }
+        if (__popc(s.m) != K) exact_set(s);                      // scores tie at the threshold
+        in_s[0] = ((s.m >> lane) & 1u) != 0u;
+        was_in[0] = ((cr.cache >> lane) & 1u) != 0u;
+        nD = __popc(s.m & ~cr.cache);
+        const int over = cr.count + nD - C;
+        update_mask(cr, over > 0 ? word(0) : 0u, s.m, over, lane);
+        cr.count = over > 0 ? C : cr.count + nD;
+    } else {
+        uint32_t counts;
+        if (POL == CRC_POLICY_SPATIO_LRU && refine) {
+            float before[V];
 #pragma unroll
-        for (int v = 0; v < V; ++v)
-            if ((loaded >> v) & 1u) aux[v] = t;
-    }
-    // native Top-K on p^R: given as a set, or popped in rank order when the
-    // trace wants the order
-    uint32_t sel = sel_in;
-    int my_topk = 0;
-    if (!have_sel) {
-        KeyList<V> P;
+            for (int v = 0; v < V; ++v) before[v] = cr.out[v];
+            pro = scan_refine<V, ALL_VALID>(cr, pS, valid, lane, C, a.s.R, s, &counts);
+            if (pro > 0) {
+#pragma unroll
+                for (int v = 0; v < V; ++v)
+                    if (before[v] > cr.out[v]) aux[v] = t;           // came in
+            }
+        } else {
+            counts = warp_count(__fadd_rn(miss_count<V>(cr, s), kCount0));
+        }
+        if ((counts >> 6) != (uint32_t)K) {                          // scores tie at the threshold
+            exact_set(s);
+            counts = warp_count(__fadd_rn(miss_count<V>(cr, s), kCount0));
+        }
+        nD = (int)(counts & 63u);
+        // demand loads; a full cache evicts the lowest priorities outside S (they
+        // do not change while the access inserts, and inserted experts are in S)
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-            P.k[v] = is_valid(v) ? pkey(pR[v]) : 0u;
-            P.s[v] = v;
+            in_s[v] = s.s[v] != 0.f;
+            was_in[v] = cr.out[v] == 0.f;
         }
-        presort<V>(P);
-        sel = 0u;
-        for (int k = 0; k < K; ++k) {
-            uint32_t kk, slot = 0u;
-            const int owner = warp_pop_first<V>(P, lane, kk, slot);
-            if (lane == owner) sel |= 1u << slot;
-            if (topk_out) {
-                const int e = __shfl_sync(kFull, lane * V + (int)slot, owner);
-                if (lane == k) my_topk = e;
-            }
-        }
-    }
-    // demand loads; a full cache evicts the lowest priorities outside S (they
-    // do not change while the access inserts, and inserted experts are in S)
-    const uint32_t dem = sel & ~cr.cache;
-    const uint32_t hit = sel & cr.cache;
-    const int nD = (int)__reduce_add_sync(kFull, (uint32_t)__popc(dem));
-    const int freeslots = C - cr.count;
-    if (nD > freeslots) {
-        uint32_t kV[V];
+        const int over = cr.count + nD - C;
+        if (over > 0) {
+            float key[V];
+            // Integer priorities tie all the time (experts last used at the same
+            // token), so while they fit (none exceeds the token index) the
+            // expert's position from the end goes below them: distinct keys in the
+            // same order, below 2^126 as bits of a float.
+            if (POL != CRC_POLICY_LRFU && t < (1u << 22)) {
 #pragma unroll
-        for (int v = 0; v < V; ++v)
-            kV[v] = POL == CRC_POLICY_LRFU
-                        ? __float_as_uint(__fmul_rn(cr.aT[v], lrfu_decay(a.lambda2, t - aux[v])))
-                        : aux[v];
-        uint32_t vset = cr.cache & ~sel;
-        for (int i = 0; i < nD - freeslots; ++i) {
-            uint32_t kv, vslot = 0u;
-            const int vo = warp_last_member<V>(kV, vset, lane, kv, vslot);
-            const uint32_t rm = (lane == vo) ? (1u << vslot) : 0u;
-            vset &= ~rm;
-            cr.cache &= ~rm;
+                for (int v = 0; v < V; ++v)
+                    key[v] = __uint_as_float((aux[v] << 8) | (255u - (uint32_t)(lane * V + v)));
+                update_cache<V, KeyTies::kNone>(cr, key, s, over, C - K, lane);
+            } else {
+                // (aux above 2^126's bits would need 2 billion tokens)
+#pragma unroll
+                for (int v = 0; v < V; ++v) key[v] = __uint_as_float(word(v));
+                update_cache<V, KeyTies::kOften>(cr, key, s, over, C - K, lane);
+            }
+            cr.count = C;
+        } else {
+#pragma unroll
+            for (int v = 0; v < V; ++v) cr.out[v] = __fmaf_rn(-s.s[v], cr.out[v], cr.out[v]);
+            cr.count += nD;
         }
-        cr.count = C;
-    } else {
-        cr.count += nD;
     }
-    cr.cache |= dem;
     // the selected experts' priorities after the access
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        if (!((sel >> v) & 1u)) continue;
-        const bool h = (hit >> v) & 1u;
+        if (!in_s[v]) continue;
+        const bool h = was_in[v];
         if constexpr (POL == CRC_POLICY_LFU) {
             aux[v] = h ? aux[v] + 1u : 1u;
         } else if constexpr (POL == CRC_POLICY_LRFU) {
@@ -133,7 +146,6 @@ __device__ __forceinline__ void policy_step(ChainRegs<V>& cr, uint32_t (&aux)[V]
     cr.hits += (uint32_t)(K - nD);
     cr.misses += (uint32_t)nD;
     cr.pro += (uint32_t)pro;
-    if (topk_out && lane < K) topk_out[lane] = (uint8_t)my_topk;
     if (lane == 0) {
         if (miss_out) *miss_out = (uint8_t)nD;
         if (pro_out) *pro_out = (uint8_t)pro;
@@ -143,8 +155,6 @@ __device__ __forceinline__ void policy_step(ChainRegs<V>& cr, uint32_t (&aux)[V]
 template <int V, bool ALL_VALID, int KP, int POL>
 __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWarps)
     cache_scan_policy_kernel(PolicyArgs pa) {
-    // Top-K sets of the next 32 tokens of each warp's chain, one row per token
-    __shared__ uint32_t sel_s[kScanWarps][32][8];
     const ScanArgs& a = pa.s;
     StateHeader* hdr = reinterpret_cast<StateHeader*>(a.state);
     const StateLayout lay = state_layout(a.B, a.L, a.N);
@@ -175,8 +185,9 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
 
         ChainState& cs = chains[chain];
         ChainRegs<V> cr;
-        cr.cache = lane_bits<V>(cs.bits, lane, N);
-        cr.count = (int)__reduce_add_sync(kFull, (uint32_t)__popc(cr.cache));
+        const uint32_t resident = lane_bits<V>(cs.bits, lane, N);
+        cr.set_bits(resident);
+        cr.count = (int)__reduce_add_sync(kFull, (uint32_t)__popc(resident));
         uint32_t aux[V];
         {
             Vec<V> x = load_vec<V>(val + (size_t)chain * N + lane * V, has);
@@ -188,72 +199,77 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
         }
         cr.hits = cr.misses = cr.pro = 0u;
 
-        const float* base = a.scores + lane * V;
-        auto unit_ptr = [&](int t, int ll) -> const float* {
-            return base + (((size_t)b * T + t) * L + ll) * row;
-        };
+        // running pointer to this lane's part of unit (b, t, l); p^S of rho(t, l)
+        // at a fixed offset, the carry for the first token of layer 0
+        const float* row0 = a.scores + ((size_t)b * T * L + l) * row;       // token 0 of the chain
         const float* carry_in = carry + ((size_t)parity * a.B + b) * N + lane * V;
-        auto pred_ptr = [&](int t) -> const float* {     // p^S of rho(t, l)
-            if (l > 0) return unit_ptr(t, l - 1) + 2 * N;
-            if (t > 0) return unit_ptr(t - 1, L - 1) + 2 * N;
-            return carry_in;
-        };
-        const bool want_s = POL == CRC_POLICY_SPATIO_LRU && a.R > 0;
-        // without a rank-order trace the Top-K set is taken for 32 tokens at
-        // a time, lane j for token t + j (it does not depend on the cache)
-        const bool batch_sel = a.trace_topk == nullptr;
-        uint32_t (*sel_rows)[8] = sel_s[(threadIdx.x >> 5) % kScanWarps];
-        const float* row_base = a.scores + ((size_t)b * T * L + l) * row;   // token 0 of chain
-        // running pointer to unit (b, t, l); p^S of rho(t, l) at a fixed offset
         const size_t tok = (size_t)L * row;
         const ptrdiff_t s_off = l > 0 ? (ptrdiff_t)2 * N - (ptrdiff_t)row
                                       : (ptrdiff_t)(L - 1) * (ptrdiff_t)row - (ptrdiff_t)tok +
                                             (ptrdiff_t)2 * N;
-        const float* up = unit_ptr(0, l);
-        const bool traced = a.trace_topk || a.trace_miss || a.trace_pro;
+        const bool want_s = POL == CRC_POLICY_SPATIO_LRU && a.R > 0;
+        const bool rank_order = a.trace_topk != nullptr;
 
-        Vec<V> cR = load_vec<V>(up, has);
-        Vec<V> cS = load_vec<V>(pred_ptr(0), has && want_s && t0 >= 1);
-        for (int t = 0; t < T; ++t) {
-            if (batch_sel && (t & 31) == 0) {
-                __syncwarp();
-                if (t + lane < T)
-                    row_topk_mask<KP>(row_base + (size_t)(t + lane) * tok, N, a.K, sel_rows[lane]);
-                __syncwarp();
+        // the rows pass through a ring in shared memory (ring_copy)
+        constexpr int D = scan_ahead<V>();
+        constexpr int ROWS = POL == CRC_POLICY_SPATIO_LRU ? 2 : 1;
+        __shared__ __align__(16) float ring[kScanWarps][D][ROWS][32 * V];
+        float (*mine)[ROWS][32 * V] = ring[(threadIdx.x >> 5) % kScanWarps];
+        if (!has) {                              // slots past N read as 0
+#pragma unroll
+            for (int i = 0; i < D * ROWS; ++i)
+#pragma unroll
+                for (int v = 0; v < V; ++v) mine[i / ROWS][i % ROWS][lane * V + v] = 0.f;
+        }
+        const float* up = row0 + lane * V;
+        auto load = [&](int t) {                 // t: the token `up` points at
+            if (t < T && has) {
+                ring_copy<V>(&mine[t % D][0][lane * V], up);
+                if (want_s && t0 + t >= 1)
+                    ring_copy<V>(&mine[t % D][ROWS - 1][lane * V],
+                                 l == 0 && t == 0 ? carry_in : up + s_off);
             }
-            uint32_t sel_in = 0u;
-            if (batch_sel && has) {
-                const uint32_t e0 = (uint32_t)lane * V;
-                sel_in = (sel_rows[t & 31][e0 >> 5] >> (e0 & 31)) & ((1u << V) - 1u);
-            }
-            Vec<V> nR, nS;
-            if (t + 1 < T) {
-                nR = load_vec<V>(up + tok, has);
-                nS = load_vec<V>(up + tok + s_off, has && want_s);
-            }
+            ring_commit();
             up += tok;
-            const bool refine = want_s && (t0 + t >= 1);
-            if (traced) {
-                const size_t unit = ((size_t)b * a.trace_T + a.trace_t0 + t) * L + l;
-                policy_step<V, ALL_VALID, POL>(cr, aux, cR.v, cS.v, refine, valid, lane, pa,
-                                               (uint32_t)(t0 + t), batch_sel, sel_in,
-                                          a.trace_topk ? a.trace_topk + unit * a.K : nullptr,
-                                          a.trace_miss ? a.trace_miss + unit : nullptr,
-                                          a.trace_pro ? a.trace_pro + unit : nullptr);
-            } else {
-                policy_step<V, ALL_VALID, POL>(cr, aux, cR.v, cS.v, refine, valid, lane, pa,
-                                               (uint32_t)(t0 + t), true, sel_in, nullptr,
-                                               nullptr, nullptr);
+        };
+        float theta = 0.f, th = 0.f;             // Top-K thresholds: lane j token t + j's; t's
+        auto step = [&](int t) {
+            float pR[V], pS[V];
+            ring_read<V>(&mine[t % D][0][lane * V], pR);
+            ring_read<V>(&mine[t % D][ROWS - 1][lane * V], pS);
+            if ((t & 31) == 0) {
+                if (t + lane < T)
+                    theta = row_theta_k<KP>(row0 + (size_t)(t + lane) * tok, N, a.K);
+                th = __shfl_sync(kFull, theta, 0);
             }
-            cR = nR;
-            cS = nS;
+            Sel<V> s;
+            const size_t unit = ((size_t)b * a.trace_T + a.trace_t0 + t) * L + l;
+            if (rank_order)
+                sel_from_bits<V>(
+                    topk_ranked<V>(pR, valid, lane, a.K, a.trace_topk + unit * a.K), s);
+            else
+                sel_above<V, ALL_VALID>(pR, th, valid, s);
+            policy_step<V, ALL_VALID, POL>(
+                cr, aux, pR, pS, want_s && t0 + t >= 1, valid, lane, pa, (uint32_t)(t0 + t),
+                s, [&](Sel<V>& x) { sel_ties<V>(pR, valid, lane, a.K, x); },
+                a.trace_miss ? a.trace_miss + unit : nullptr,
+                a.trace_pro ? a.trace_pro + unit : nullptr);
+        };
+#pragma unroll
+        for (int t = 0; t < D - 1; ++t) load(t);
+#pragma unroll 1
+        for (int t = 0; t < T; ++t) {
+            load(t + D - 1);
+            ring_wait<D - 1>();                  // token t's copies have landed
+            step(t);
+            th = __shfl_sync(kFull, theta, (t + 1) & 31);
         }
 
         // write back the chain
         const int NW = (N + 31) >> 5;
         for (int w = 0; w < NW; ++w) {
             const int e0 = lane * V;
-            const uint32_t contrib = (has && (e0 >> 5) == w) ? (cr.cache << (e0 & 31)) : 0u;
+            const uint32_t contrib = (has && (e0 >> 5) == w) ? (cr.bits(lane) << (e0 & 31)) : 0u;
             const uint32_t word = __reduce_or_sync(kFull, contrib);
             if (lane == 0) cs.bits[w] = word;
         }
@@ -272,7 +288,7 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
         }
         // the last layer hands its final p^S to layer 0 of the next call
         if (l == L - 1 && has) {
-            const float* src = unit_ptr(T - 1, L - 1) + 2 * N;
+            const float* src = row0 + lane * V + (size_t)(T - 1) * tok + 2 * N;
             float* dst = carry + ((size_t)(parity ^ 1u) * a.B + b) * N + lane * V;
 #pragma unroll
             for (int v = 0; v < V; ++v)

@@ -1,0 +1,70 @@
+"""The scan kernels' paths that ordinary inputs rarely or never take, against
+the oracle's literal scans: scores that tie at the Top-K threshold, in the
+refinement and in the evictions (the general forms), scores far above
+probabilities, and comparison-policy states whose token counter has passed the
+range in which priority and expert index share a word.
+"""
+import numpy as np
+import pytest
+
+import crc_synth as S
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def C():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2609_04895_gb300 import build
+    build.build()
+    from paper_2609_04895_gb300 import crc
+    crc.load()
+    return crc
+
+
+def scores(w, seed, levels, scale=1.0):
+    """Scores on a few levels (many ties), fp32, sums exact."""
+    r = np.random.default_rng(seed)
+    x = r.integers(0, levels, (w.B, w.T, w.L, 3, w.N)).astype(np.float32) / levels
+    return np.ascontiguousarray(x * np.float32(scale))
+
+
+@pytest.mark.parametrize("N,K,C_,R", [(16, 3, 5, 2), (32, 4, 8, 4), (48, 8, 8, 8), (64, 6, 16, 3),
+                                      (128, 8, 32, 4), (128, 8, 9, 16), (256, 32, 40, 6)])
+@pytest.mark.parametrize("levels,scale", [(4, 1.0), (64, 1.0), (100000, 1.0), (64, 2.0 ** 126)])
+def test_scan_ties_and_scales(C, oracle_lib, N, K, C_, R, levels, scale):
+    w = S.TINY.with_(N=N, K=K, C=C_, R=R, B=2, T=40, L=3)
+    x = scores(w, 5, levels, scale)
+    o = oracle_lib.scan(x, K, C_, R, trace=False)
+    p = C.problem_of(w)
+    st = C.State(p)
+    C.cache_scan(p, torch.from_numpy(x).cuda(), st, None)
+    g = st.read(want_caches=True, want_retention=True, want_chain_counters=True)
+    assert np.array_equal(g["cache_bits"], o["cache_bits"])
+    assert np.array_equal(g["chain_counters"], o["counters"])
+    assert np.array_equal(g["retention"].view(np.uint32), o["aT"].view(np.uint32))
+
+
+@pytest.mark.parametrize("policy", ["lru", "lfu", "spatio_lru"])
+@pytest.mark.parametrize("N,K,C_", [(16, 2, 4), (128, 8, 32), (256, 8, 20)])
+def test_policy_priorities_past_the_packed_range(C, policy, N, K, C_):
+    """A state whose token counter crosses 2^22 decides as one that starts at
+    token 1 (the policies depend on differences of token indices only)."""
+    w = S.TINY.with_(N=N, K=K, C=C_, R=2, B=2, T=48, L=3)
+    x = torch.from_numpy(scores(w, 9, 512)).cuda()
+    p = C.problem_of(w)
+    out = []
+    for t0 in (1, (1 << 22) - 24):
+        st = C.State(p)
+        head = st.buf[:256].view(torch.int64)
+        head[1] = t0                                   # the header's token counter
+        st.buf[:256].view(torch.int32)[14] = C.POLICIES[policy]     # and its policy
+        tr = C.Trace.alloc(p, w.T)
+        C.cache_scan_policy(p, x, st, policy, tr)
+        g = st.read(want_caches=True, want_chain_counters=True)
+        out.append((g["cache_bits"], g["chain_counters"], tr.misses.cpu().numpy(),
+                    tr.proactive.cpu().numpy()))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
