@@ -281,15 +281,19 @@ int crc_route_and_cache(const crc_problem* p, const uint16_t* hidden_dev,
     if (!workspace_dev || !aligned(workspace_dev, 256)) return CRC_EINVAL;
     if ((rc = check_trace(trace))) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // the fused kernel knows the Top-K as a set only: a trace in rank order
+    // the scores of one token have to fit, unless the fused kernel's ring does
+    const size_t per_token = crc_workspace_bytes(p, 1);
+    const long long fit = (long long)(workspace_bytes / per_token);
+    if (fit < 1 && workspace_bytes < fused_workspace_bytes(*p)) return CRC_EINVAL;
+    // the fused kernels know the Top-K as a set only: a trace in rank order
     // takes the two-kernel path
     if (!(trace && trace->topk_dev)) {
+        rc = launch_short(*p, hidden_dev, w_cat_dev, T, state_dev, trace, s);
+        if (rc != CRC_EUNSUPPORTED) return rc;
         rc = launch_fused(*p, hidden_dev, w_cat_dev, T, state_dev, workspace_dev, workspace_bytes,
                           trace, s);
         if (rc != CRC_EUNSUPPORTED) return rc;
     }
-    const size_t per_token = crc_workspace_bytes(p, 1);
-    const long long fit = (long long)(workspace_bytes / per_token);
     if (fit < 1) return CRC_EINVAL;
     const int chunk = fit < T ? (int)fit : T;
     float* scores = static_cast<float*>(workspace_dev);

@@ -295,10 +295,10 @@ struct ChainRegs {
     uint32_t hits, misses, pro;
 
     __device__ __forceinline__ uint32_t bits(int) const {    // the residency as V bits
-        uint32_t b = 0u;
+        float b = kCount0 + (float)((1 << V) - 1);
 #pragma unroll
-        for (int v = 0; v < V; ++v) b |= out[v] == 0.f ? 1u << v : 0u;
-        return b;
+        for (int v = 0; v < V; ++v) b = __fmaf_rn(out[v], -(float)(1 << v), b);
+        return __float_as_uint(b) & ((1u << V) - 1u);
     }
     __device__ __forceinline__ void set_bits(uint32_t b) {
 #pragma unroll
@@ -858,10 +858,10 @@ __device__ __forceinline__ uint32_t sel_bits(const Sel<V>& sel, int lane) {
     if constexpr (V == 1) {
         return (sel.m >> lane) & 1u;
     } else {
-        uint32_t b = 0u;
+        float b = kCount0;
 #pragma unroll
-        for (int v = 0; v < V; ++v) b |= sel.s[v] != 0.f ? 1u << v : 0u;
-        return b;
+        for (int v = 0; v < V; ++v) b = __fmaf_rn(sel.s[v], (float)(1 << v), b);
+        return __float_as_uint(b) & ((1u << V) - 1u);
     }
 }
 

@@ -29,7 +29,8 @@ struct StateHeader {           // 256 bytes at offset 0
     int32_t L, N, K, C, R, B;  // the problem this state was made for
     uint64_t expert_bytes;
     uint32_t policy;           // 0: the method; else the comparison policy that owns the state
-    uint32_t pad[49];
+    uint32_t aborted;          // a wait of the running short call ran out
+    uint32_t pad[48];
 };
 static_assert(sizeof(StateHeader) == 256, "header size");
 
@@ -381,6 +382,15 @@ __device__ __forceinline__ void tmem_ld16f(uint32_t taddr, float* v) {
         : "r"(taddr));
 }
 
+// 32 lanes x 8 consecutive 32-bit columns, written straight into v.
+__device__ __forceinline__ void tmem_ld8f(uint32_t taddr, float* v) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+          "=f"(v[7])
+        : "r"(taddr));
+}
+
 // 32 lanes x 32 / 16 consecutive 32-bit columns stored from registers.
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float* v) {
     asm volatile(
@@ -415,6 +425,17 @@ __device__ __forceinline__ void pin16(float* z) {
                  : "+f"(z[0]), "+f"(z[1]), "+f"(z[2]), "+f"(z[3]), "+f"(z[4]), "+f"(z[5]),
                    "+f"(z[6]), "+f"(z[7]), "+f"(z[8]), "+f"(z[9]), "+f"(z[10]), "+f"(z[11]),
                    "+f"(z[12]), "+f"(z[13]), "+f"(z[14]), "+f"(z[15]));
+}
+
+__device__ __forceinline__ void pin8(float* z) {
+    asm volatile(""
+                 : "+f"(z[0]), "+f"(z[1]), "+f"(z[2]), "+f"(z[3]), "+f"(z[4]), "+f"(z[5]),
+                   "+f"(z[6]), "+f"(z[7]));
+}
+
+// Barrier `id` (1..15) of the CTA among `threads` threads.
+__device__ __forceinline__ void named_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 // TMA tensor store (5-D), bulk-group completion.
