@@ -15,9 +15,8 @@
 // Reductions: the fp32 bit patterns of the (non-negative) scores are ordered
 // like the scores, so a warp-wide extreme is a lane-local extreme and one
 // redux.sync; the slot that holds it finds itself by comparing, and a count of
-// the holders proves that there was exactly one.  Two holders (equal scores),
-// and a cache that is still filling, go to the general forms, which settle
-// every case by expert index with ballots.
+// the holders proves that there was exactly one.  Two holders (equal scores) go
+// to the general forms, which settle every case by expert index with ballots.
 //
 // What bounds the step: the integer pipe (16 lanes a scheduler) when many
 // chains share an SM, and for a few chains the latency of some 300 dependent
@@ -510,8 +509,7 @@ __device__ __forceinline__ float row_theta_k(const float* row, int N, int K) {
 // the strict test, ending the pass exactly as the rank test or the strict
 // test ends it here.
 //
-// The general form, for a cache that is filling and for ties (keys: score bits,
-// 0 in invalid slots).  A function of its own, so the scans' loops stay short.
+// The general form, for ties (keys: score bits, 0 in invalid slots).  A function of its own, so the scans' loops stay short.
 // Returns the cache (V bits) | its count << 8 | the proactive loads << 20.
 template <int V>
 __device__ __noinline__ uint32_t refine_general(Keys<V> key, uint32_t cache, int count,
@@ -576,14 +574,14 @@ __device__ __forceinline__ float miss_count(const ChainRegs<V>& cr, const Sel<V>
     return __fmaf_rn(all, 64.f, miss);
 }
 
-// The refinement with a full cache (every access but the first few): a round
-// takes the best non-resident's score and the lowest resident's in two
-// independent reductions, then one count that carries both c's rank and the
-// demand misses of the native Top-K s against the cache as it stands, so the
-// round that ends the pass has also counted them.  A swap is made by the
-// slots that hold the two scores, after a count has shown that each has one
-// holder, c's among all experts and the lowest's among the residents;
-// otherwise refine_general takes the pass on from the cache as it is.
+// The refinement: a round takes the best non-resident's score and the lowest
+// resident's in two independent reductions, then one count that carries both
+// c's rank and the demand misses of the native Top-K s against the cache as it
+// stands, so the round that ends the pass has also counted them.  A load or a
+// swap is made by the slots that hold the two scores, after a count has shown
+// that each has one holder, c's among all experts and the lowest's among the
+// residents; otherwise refine_general takes the pass on from the cache as it
+// is.
 // *counts receives the demand misses and, above bit 6, the members of s.
 template <int V, bool ALL_VALID>
 __device__ __forceinline__ int scan_refine(ChainRegs<V>& cr, const float (&pS)[V], uint32_t valid,
@@ -596,41 +594,42 @@ __device__ __forceinline__ int scan_refine(ChainRegs<V>& cr, const float (&pS)[V
         if (!ALL_VALID && !((valid >> v) & 1u)) k[v] = 0.f;
     }
     int pro = 0;
-    bool general = cr.count < C;
-    if (!general) {
+    bool general = false;
 #pragma unroll 1
-        while (true) {
-            float x[V], y[V];
+    while (true) {
+        const bool full = cr.count == C;
+        float x[V], y[V];
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-                x[v] = __fmul_rn(k[v], cr.out[v]);                 // invalid slots: 0
-                y[v] = __fmaf_rn(cr.out[v], kFar, k[v]);
-            }
-            const float mx = warp_max_f(lane_max_f<V>(x));
-            const float mn = warp_min_f(lane_min_f<V>(y));
-            float gt = kCount0;
-#pragma unroll
-            for (int v = 0; v < V; ++v) gt = __fadd_rn(gt, set_gt(k[v], mx));
-            const uint32_t tot = warp_count(__fmaf_rn(miss_count<V>(cr, s), 1024.f, gt));
-            *counts = tot >> 10;
-            // not among the top R, or no higher than the lowest resident: neither
-            // is any later candidate
-            if ((int)(tot & 1023u) >= R || __float_as_uint(mx) <= __float_as_uint(mn)) break;
-            float h = kCount0, in[V], go[V];
-#pragma unroll
-            for (int v = 0; v < V; ++v) {
-                in[v] = set_eq(k[v], mx);
-                go[v] = set_eq(y[v], mn);
-                h = __fadd_rn(h, in[v]);
-                h = __fmaf_rn(go[v], 1024.f, h);
-            }
-            general = warp_count(h) != 1025u || mn >= kFar;
-            if (general) break;
-#pragma unroll
-            for (int v = 0; v < V; ++v)
-                cr.out[v] = __fadd_rn(__fsub_rn(cr.out[v], in[v]), go[v]);
-            ++pro;
+        for (int v = 0; v < V; ++v) {
+            x[v] = __fmul_rn(k[v], cr.out[v]);                 // invalid slots: 0
+            y[v] = __fmaf_rn(cr.out[v], kFar, k[v]);
         }
+        const float mx = warp_max_f(lane_max_f<V>(x));
+        const float mn = warp_min_f(lane_min_f<V>(y));
+        float gt = kCount0;
+#pragma unroll
+        for (int v = 0; v < V; ++v) gt = __fadd_rn(gt, set_gt(k[v], mx));
+        const uint32_t tot = warp_count(__fmaf_rn(miss_count<V>(cr, s), 1024.f, gt));
+        *counts = tot >> 10;
+        // not among the top R, or no higher than the lowest resident of a full
+        // cache: neither is any later candidate
+        if ((int)(tot & 1023u) >= R || (full && __float_as_uint(mx) <= __float_as_uint(mn))) break;
+        const float lowest = full ? mn : -1.f;                 // who leaves; nobody
+        float h = kCount0, in[V], go[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            in[v] = set_eq(k[v], mx);
+            go[v] = set_eq(y[v], lowest);
+            h = __fadd_rn(h, in[v]);
+            h = __fmaf_rn(go[v], 1024.f, h);
+        }
+        general = warp_count(h) != (full ? 1025u : 1u) || mn >= kFar || mx == 0.f;
+        if (general) break;
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+            cr.out[v] = __fadd_rn(__fsub_rn(cr.out[v], in[v]), go[v]);
+        cr.count += full ? 0 : 1;
+        ++pro;
     }
     if (general) {
         Keys<V> key;
