@@ -196,7 +196,6 @@ __device__ __forceinline__ void fused_scan_role(const FusedArgs& a, uint32_t* er
     const bool want_s = a.R > 0;
     const uint32_t e0 = (uint32_t)lane * V;
     const int NW = (N + 31) >> 5;
-    const bool traced = TRACED && (a.tr_miss || a.tr_pro || a.tr_mid || a.tr_after || a.tr_sel);
     while (true) {
         uint32_t item = 0u;
         if (lane == 0) item = atomicAdd(&a.ctl[0], 1u);
@@ -301,27 +300,32 @@ __device__ __forceinline__ void fused_scan_role(const FusedArgs& a, uint32_t* er
             float T[V], S[V];
             uint32_t selw;
         };
+        // A traced item packs each lane's part of the two cache sets of four
+        // steps into a word, kept until the item's end in the lane's place of
+        // the own tile's s^T, in the first of each 4 V rows, which has been read
+        // for the last time by then.  (A word a step dirtied every line of the
+        // ring anew: 2.04 against 1.88 ms for 64 x 128 tokens of N = 128,
+        // d = 4096.)  Word of steps t .. t + 3, t a multiple of 4, of lane q:
+        auto trace_word = [&](int q, int t) {
+            const int e = q * V, r = sbi * a.TB + (t & ~(4 * V - 1));
+            return reinterpret_cast<uint32_t*>(const_cast<uint8_t*>(own) + RL::ST) +
+                   ((size_t)(e >> 2) * 128 + r) * 4 + (e & 3) + ((t >> 2) & (V - 1));
+        };
+        uint32_t packed = 0u;
         auto step = [&](int tbi, const In& q) {
             if ((tbi & 7) == 0) prefetch_rows(tbi + 24);
             Sel<V> s;
             sel_from_bits<V>(q.selw >> (e0 & 31), s);
-            const bool tr = traced && CRC_IN_BOUNDS(tb * a.TB + tbi < a.T, err);
-            const size_t unit = ((size_t)b * a.T + tb * a.TB + tbi) * L + l;
             int nD;
-            const int pro = scan_apply<V, ALL_VALID>(
+            uint32_t mid = 0u;
+            scan_apply<V, ALL_VALID>(
                 cr, q.T, q.S, want_s && tbi >= refine_from, valid, lane, a.K, a.C, a.R, s, &nD,
-                [](Sel<V>&) {},
-                [&] {
-                    if (tr && a.tr_mid)
-                        store_cache_words<V>(cr.bits(lane), lane, N, a.tr_mid + unit * NW);
-                });
-            if (tr) {
-                if (a.tr_after) store_cache_words<V>(cr.bits(lane), lane, N, a.tr_after + unit * NW);
-                if (a.tr_sel && has && (e0 & 31u) == 0u) a.tr_sel[unit * NW + (e0 >> 5)] = q.selw;
-                if (lane == 0) {
-                    if (a.tr_miss) a.tr_miss[unit] = (uint8_t)nD;
-                    if (a.tr_pro) a.tr_pro[unit] = (uint8_t)pro;
-                }
+                [](Sel<V>&) {}, [&] { if (TRACED) mid = cr.bits(lane); });
+            if constexpr (TRACED) {
+                packed = (packed >> 8) | (mid << 24) | (cr.bits(lane) << (24 + V));
+                const bool last = tbi + 1 == steps;
+                if (has && ((tbi & 3) == 3 || last))
+                    *trace_word(lane, tbi & ~3) = packed >> (8 * (3 - (tbi & 3)));
             }
             // debug builds: every expert the step made resident lies in this
             // lane's range and the cache holds at most C experts
@@ -334,6 +338,57 @@ __device__ __forceinline__ void fused_scan_role(const FusedArgs& a, uint32_t* er
             if (tbi + 1 < steps) fetch(tbi + 1, next.T, next.S, next.selw);
             step(tbi, q);
             q = next;
+        }
+        if constexpr (TRACED) {
+            // The item's trace, a row a lane: the sets' words, the misses |S \ C~|
+            // and the proactive loads |C~ \ C|, with C the cache of the row
+            // before (an expert the refinement loads stays until its end).
+            // Gathering each step's sets over the warp as the chain went took a
+            // third of a traced step: 0.93 against 0.61 us a token untraced.
+            __syncwarp();
+            uint32_t before[RL::NW];               // the cache before this lane's row
+#pragma unroll
+            for (int w = 0; w < RL::NW; ++w) before[w] = __ldcg(&cs.bits[w]);
+            for (int i0 = 0; i0 < steps; i0 += 32) {
+                const int i = imin(i0 + lane, steps - 1);
+                const bool wr = i0 + lane < steps && CRC_IN_BOUNDS(tb * a.TB + i < a.T, err);
+                const int r = sbi * a.TB + i;
+                const size_t unit = ((size_t)b * a.T + tb * a.TB + i) * L + l;
+                int nD = 0, pro = 0;
+#pragma unroll
+                for (int w = 0; w < RL::NW; ++w) {
+                    constexpr int PER = imin(NH, 32) / V;        // lanes to a word
+                    constexpr uint32_t ONES = (1u << V) - 1u;
+                    const uint32_t sel = __ldcg(
+                        reinterpret_cast<const uint32_t*>(own + RL::SEL) + (size_t)w * 128 + r);
+                    uint32_t mw = 0u, aw = 0u;
+#pragma unroll
+                    for (int c0 = 0; c0 < PER; c0 += 8) {
+                        uint32_t x[8];
+#pragma unroll
+                        for (int c = 0; c < 8; ++c)
+                            x[c] = __ldcg(trace_word(w * (32 / V) + c0 + c, i & ~3)) >> (8 * (i & 3));
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            mw |= (x[c] & ONES) << ((c0 + c) * V);
+                            aw |= ((x[c] >> V) & ONES) << ((c0 + c) * V);
+                        }
+                    }
+                    // the cache before: the row before's, the last row's of the
+                    // round before for lane 0
+                    const uint32_t up = __shfl_up_sync(kFull, aw, 1);
+                    const uint32_t was = lane == 0 ? before[w] : up;
+                    before[w] = __shfl_sync(kFull, aw, 31);
+                    nD += __popc(sel & ~mw);
+                    pro += __popc(mw & ~was);
+                    if (wr && a.tr_mid) a.tr_mid[unit * NW + w] = mw;
+                    if (wr && a.tr_after) a.tr_after[unit * NW + w] = aw;
+                    if (wr && a.tr_sel) a.tr_sel[unit * NW + w] = sel;
+                }
+                if (wr && a.tr_miss) a.tr_miss[unit] = (uint8_t)nD;
+                if (wr && a.tr_pro) a.tr_pro[unit] = (uint8_t)pro;
+            }
+            __syncwarp();
         }
         // the last layer hands p^S of the call's last token to layer 0 of the next call
         if (l == L - 1 && want_s && tb * a.TB + a.TB >= a.T && steps > 0 && has) {
