@@ -118,6 +118,8 @@ EXPORTS = [
 def load(path: str = LIB_PATH):
     """Load libcrc.so (built by paper_2609_04895_gb300.build); raises if absent."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(path):
@@ -139,8 +141,10 @@ def _ck(rc: int, what: str):
 
 def _stream(stream) -> int:
     if stream is None:
+        # the current stream's handle without the Stream object around it, which
+        # took 3 of a one-token call's 13 us on the host
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -493,14 +497,14 @@ def cache_loss(p: crc_problem, probs, top_b: int, tau: float, w_T: float = 1.0,
 
 def route_and_cache(p: crc_problem, hidden, w_cat, state: State, trace: Trace | None = None,
                     workspace=None, stream=None):
-    import torch
-    T = hidden.shape[1]
+    T = hidden.size(1)
     if workspace is None:
+        import torch
         workspace = torch.empty(crc_workspace_bytes(p, T), dtype=torch.uint8,
                                 device=hidden.device)
-    crc_route_and_cache(p, hidden.data_ptr(), w_cat.data_ptr(), T, state.ptr, state.nbytes,
-                        None if trace is None else trace.c(), workspace.data_ptr(),
-                        workspace.numel() * workspace.element_size(), stream)
+    crc_route_and_cache(p, hidden.data_ptr(), w_cat.data_ptr(), T, state.buf.data_ptr(),
+                        state.nbytes, None if trace is None else trace.c(),
+                        workspace.data_ptr(), workspace.nbytes, stream)
     return workspace
 
 
