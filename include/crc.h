@@ -221,10 +221,11 @@ size_t crc_workspace_bytes(const crc_problem *p, int32_t chunk_tokens);
 
 /* Workspace bytes with which crc_route_and_cache runs as ONE fused kernel
  * (router heads on the tensor cores and the scan together; the router scores
- * then only pass through a ring of tiles in the workspace).  The fused kernel
- * serves calls with K <= 8 and 16 <= N <= 128 whose trace, if any, does not
+ * then only pass through a ring of tiles in the workspace).  The fused kernels
+ * serve calls with K <= 8 and 16 <= N <= 128 whose trace, if any, does not
  * ask for the Top-K in rank order (crc_trace.topk_dev); other calls, or
- * smaller workspaces, take the chunked two-kernel path.  0 if p is invalid. */
+ * longer ones with a smaller workspace, take the chunked two-kernel path.  0 if
+ * p is invalid. */
 size_t crc_fused_workspace_bytes(const crc_problem *p);
 
 /* The whole step of the paper's decoding loop over T tokens: the router
@@ -234,16 +235,18 @@ size_t crc_fused_workspace_bytes(const crc_problem *p);
  * crc_cache_scan (bit for bit).
  * hidden_dev bf16 [B][T][L][d]; w_cat_dev bf16 [L][3N][d] (the S head is
  * not computed when R = 0).  The router scores never leave the workspace.
- * With workspace_bytes >= crc_fused_workspace_bytes(p), K <= 8 and a trace
- * that leaves topk_dev NULL (or no trace) the call is one fused kernel; for N = 128 with 128-token tiles of one stream
- * (T > 64) and an even stream count its GEMM runs on CTA pairs (clusters of
- * two, tcgen05 cta_group::2), otherwise one CTA per tile, with the same
+ * With K <= 8 and a trace that leaves topk_dev NULL (or no trace), short calls
+ * (one or two tokens, up to 64 when few enough) run as one kernel that uses no
+ * workspace, and with workspace_bytes >= crc_fused_workspace_bytes(p) the others
+ * as one persistent fused kernel; for N = 128 with an even number of tiles a
+ * layer its GEMM runs on CTA pairs (clusters of two, tcgen05 cta_group::2),
+ * otherwise one CTA per tile.  All give the same
  * results.  The pair kernel is a cooperative cluster launch; with the
  * environment variable CRC_PLAIN_CLUSTER_LAUNCH=1 (read once per process) it
  * is launched without the cooperative attribute, for kernel profilers that
  * cannot replay cooperative cluster launches (same kernel, same grid, which
- * fits the GPU at once; a stall would end in CRC_ETIMEOUT).  Without that workspace, workspace_dev holds the scores of one
- * chunk of tokens, the chunk length being the largest that fits (at least one
+ * fits the GPU at once; a stall would end in CRC_ETIMEOUT).  Without that
+ * workspace, workspace_dev holds the scores of one chunk of tokens, the chunk length being the largest that fits (at least one
  * token must fit, see crc_workspace_bytes).  256-byte alignment for the
  * workspace. */
 int crc_route_and_cache(const crc_problem *p, const uint16_t *hidden_dev,

@@ -6,7 +6,7 @@
 // up, else written back to DRAM and read from there).
 //
 // Per CTA (one per SM, cooperative launch so that all CTAs are resident), 12 warps
-// (14 when R > 4):
+// (14 for fewer than 128 experts or without the Spatio head):
 //   warp 0      TMA producer  (hidden tile + [3N x 64] weight slab per stage)
 //   warp 1      TMEM owner, tcgen05.mma issuer
 //   warps 2..5  epilogue: per tile row (thread = row) the three softmaxes,
@@ -447,20 +447,18 @@ template <int NH, int H, bool PAIR = false>
 struct FusedCfg {
     using RC = RouterCfg<NH, H>;
     static constexpr int GEMM_WARPS = 6;
-    // Scan warps per CTA, chosen at launch from the refinement budget.  Six
-    // keep up with the GEMM when R <= 4; more of them only take issue slots
-    // from the epilogue (Qwen3-30B shape: 6 -> 4.20 ms, 7 -> 4.24, 8 -> 4.29,
-    // 10 -> 4.35; 5 and 4 fall behind the tiles, 4.36 and 4.96).  With R = 8
-    // a step has up to twice the refinement rounds and six fall behind (one
-    // 128-token chunk of the Qwen3-235B shape: 15.9 ms with 6, 15.25 with 8,
-    // 15.17 with 10; with R = 2: 14.7-15.0 with 6 or 8).  The kernel's roles
-    // do not depend on the count: every warp past the GEMM warps scans.
+    // Scan warps per CTA: as many as keep up with the tiles; more only take
+    // issue slots from the epilogue.  Three heads of 128 experts: 6 (64 x 1024
+    // tokens, 5 to 8 warps within 2 %, 4 10 % slower; R = 8 the same).  Fewer
+    // columns or no Spatio head mean shorter tiles: 8 (N = 32, 64 x 1000: 6
+    // 1483 us, 8 1361; R = 0, 48 x 777: 1714 and 1608).  The kernel's roles do
+    // not depend on the count: every warp past the GEMM warps scans.
     static constexpr int SCAN_WARPS = 6;
     static constexpr int SCAN_WARPS_WIDE = 8;
     static constexpr int THREADS = 32 * (GEMM_WARPS + SCAN_WARPS);
     static constexpr int MAX_THREADS = 32 * (GEMM_WARPS + SCAN_WARPS_WIDE);
     static int threads_for(int R) {
-        return 32 * (GEMM_WARPS + (R > 4 ? SCAN_WARPS_WIDE : SCAN_WARPS));
+        return 32 * (GEMM_WARPS + (NH == 128 && R > 0 ? SCAN_WARPS : SCAN_WARPS_WIDE));
     }
     static constexpr int B_ROWS = PAIR ? RC::NCOL / 2 : RC::NCOL;        // weight rows per CTA
     static constexpr int B_BOX_ROWS = PAIR ? RC::NCH / 2 : RC::B_BOX_ROWS;

@@ -24,16 +24,54 @@ struct FusedPlan {
     size_t slot_bytes, ctl_bytes, total;
 };
 
-// Tile = SB streams x TB tokens of one layer, TB as long as the call allows
-// (128 tokens of one stream when T >= 128).  Tiles go in the order (token
-// block, layer, stream group), so a layer's weights are fetched once per
-// token block; the ring holds three token blocks of records.  T = 0 gives the
-// largest layout.
+// A tile's 128 rows are SB streams x TB tokens of one layer.  Tiles go in the
+// order (token block, layer, stream group), so a layer's weights are fetched
+// once per token block; the ring holds three token blocks of records.
+//
+// Cost of a tile by its tokens, against one of 128 tokens: a shorter block means
+// a smaller ring, whose records are read (and their lines overwritten) while
+// they are still in L2, and shorter scan items; but the weights are fetched
+// more often.  Measured, us: N = 32, 64 x 1000 tokens, TB = 128 1532, 64 1475,
+// 32 1430, 16 1361; N = 64, 40 x 600 568, 561, 561 (of fewer tiles), 625;
+// N = 128, 64 x 1024 3970, 3916, 4088; R = 0, 48 x 777 1645 (336 tiles a
+// layer), 1608 (312), 1684 (300).
+inline double tile_cost(int N, int R, int tb) {
+    const int i = tb == 128 ? 0 : tb == 64 ? 1 : tb == 32 ? 2 : 3;
+    static const double cost[4][4] = {{1.0, 0.96, 0.93, 0.90},     // N <= 32
+                                      {1.0, 0.99, 1.04, 1.15},     // N = 64
+                                      {1.0, 0.985, 1.01, 1.07},    // N = 128
+                                      {1.0, 1.05, 1.15, 1.25}};    // N = 128, R = 0
+    return cost[N <= 32 ? 0 : N <= 64 ? 1 : R > 0 ? 2 : 3][i];
+}
+
+// Tokens of a block: all of a shorter call; otherwise the cheapest by tiles a
+// layer times a tile's cost, an N = 128 plan whose tiles do not pair up (see
+// launch_fused_pair) counting 12 % more.  With fewer chains than about the scan
+// warps (1,024), or rows short enough that a tile's GEMM takes less than its
+// scan (d < 1024), the chains' steps bound the call, not its tiles, and longer
+// items are better (N = 16, d = 256, 256 x 500: 327 us, with TB = 16 358).
+// T = 0 gives the largest layout.
+inline int block_tokens(const crc_problem& p, int T) {
+    int tb = 128;
+    if (T > 0 && T <= 64)
+        while (tb > 1 && tb / 2 >= T) tb >>= 1;
+    if (T <= 64 || p.d < 1024 || (long long)p.B * p.L < 1024) return tb;
+    double best = 0.0;
+    for (int c = 128; c >= 16; c >>= 1) {
+        const int n_bg = (p.B + 128 / c - 1) / (128 / c);
+        double cost = (double)n_bg * ((T + c - 1) / c) * tile_cost(p.N, p.R, c);
+        if (p.N == 128 && n_bg % 2 != 0) cost *= 1.12;
+        if (c == 128 || cost < best) {
+            best = cost;
+            tb = c;
+        }
+    }
+    return tb;
+}
+
 inline FusedPlan fused_plan(const crc_problem& p, int T) {
     FusedPlan f;
-    int tb = 128;
-    if (T > 0)
-        while (tb > 1 && tb / 2 >= T) tb >>= 1;
+    const int tb = block_tokens(p, T);
     f.TB = tb;
     f.SB = 128 / tb;
     f.n_bg = (p.B + f.SB - 1) / f.SB;
@@ -61,7 +99,7 @@ int launch_fused_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
     using Cfg = FusedCfg<NH, H, PAIR>;
     using RC = typename Cfg::RC;
     const FusedPlan f = fused_plan(p, T);
-    if (PAIR && (f.SB != 1 || f.n_bg % 2 != 0)) return CRC_EUNSUPPORTED;
+    if (PAIR && f.n_bg % 2 != 0) return CRC_EUNSUPPORTED;
     auto kern = fused_route_cache_kernel<NH, H, V, ALL_VALID, KP, PAIR, TRACED>;
     // -1: not set up yet in this process; 0: refused; else the grid
     static int grid = -1;
