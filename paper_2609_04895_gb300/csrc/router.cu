@@ -1,10 +1,12 @@
 // Host launcher of the router-heads kernel: tensor maps, tile plan, dispatch.
 #include <cudaTypedefs.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "crc_internal.h"
 #include "router_gemm.cuh"
+#include "router_pair.cuh"
 
 namespace crc {
 
@@ -71,6 +73,59 @@ bool make_scores_map(CUtensorMap* m, float* scores, int B, int T_ext, int L, int
 
 namespace {
 
+// The launch on CTA pairs.  A layer's tiles are paired in order; an odd last
+// one has an idle partner, which costs up to half a tile's time a layer, so
+// pairs are taken when that is little or when the whole call is one wave
+// anyway.  CRC_EUNSUPPORTED: the single-CTA kernel takes the call.
+template <int H>
+int launch_router_pair(const crc_problem& p, const uint16_t* w_cat, const CUtensorMap& mh,
+                       const CUtensorMap& ms, const RouterArgs& a, cudaStream_t stream) {
+    using Cfg = RouterPairCfg<H>;
+    RouterPairArgs pa;
+    pa.r = a;
+    const int tiles = a.n_sb * a.n_tb;
+    pa.pairs_per_layer = (tiles + 1) / 2;
+    pa.num_pairs = p.L * pa.pairs_per_layer;
+    if (tiles % 2 != 0 && tiles < 9 && 2 * pa.num_pairs > sm_count()) return CRC_EUNSUPPORTED;
+    auto kern = router_pair_kernel<H>;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)(sm_count() / 2 * 2));
+    c.blockDim = dim3(Cfg::THREADS);
+    c.dynamicSmemBytes = Cfg::SMEM_BYTES;
+    c.stream = stream;
+    c.attrs = at;
+    c.numAttrs = 1;
+    // clusters that fit the GPU at once, -1 before the first call
+    static std::atomic<int> resident{-1};
+    int fit = resident.load();
+    if (fit < 0) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 Cfg::SMEM_BYTES) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&fit, (const void*)kern, &c) != cudaSuccess) {
+            (void)cudaGetLastError();
+            fit = 0;
+        }
+        resident.store(fit);
+    }
+    if (fit < 1) return CRC_EUNSUPPORTED;
+    c.gridDim = dim3((unsigned)(2 * (pa.num_pairs < fit ? pa.num_pairs : fit)));
+    CUtensorMap mw;
+    if (!make_weight_map(&mw, w_cat, p.L, 3 * Cfg::NH, p.d, Cfg::W_ROWS)) return CRC_ECUDA;
+    void* args[] = {(void*)&mh, (void*)&mw, (void*)&ms, (void*)&pa};
+    cudaError_t e;
+    {
+        ProfScope prof(CRC_KERNEL_ROUTER, stream);
+        e = cudaLaunchKernelExC(&c, (const void*)kern, args);
+    }
+    note_launch();
+    return e == cudaSuccess ? CRC_OK : CRC_ECUDA;
+}
+
 template <int NH, int H>
 int launch_router_t(const crc_problem& p, const uint16_t* hidden, int T_total, int t_begin,
                     int T_ext, const uint16_t* w_cat, float* scores, uint32_t* err,
@@ -108,6 +163,10 @@ int launch_router_t(const crc_problem& p, const uint16_t* hidden, int T_total, i
                                  Cfg::SMEM_BYTES) != cudaSuccess)
             return CRC_ECUDA;
         attr_set = true;
+    }
+    if constexpr (NH == 128) {
+        const int rc = launch_router_pair<H>(p, w_cat, mh, ms, a, stream);
+        if (rc != CRC_EUNSUPPORTED) return rc;
     }
     const int grid = a.num_tiles < sm_count() ? a.num_tiles : sm_count();
     {
