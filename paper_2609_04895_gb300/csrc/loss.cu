@@ -43,6 +43,10 @@
 namespace crc {
 namespace {
 
+// The warp-per-row kernel is bound by issue, most of it on the integer pipe at
+// half rate: theta_B's search on the FMA pipe, proved by one count instead of a
+// count a round, took 64 x 512 tokens of the Qwen3 shape from 1223 to 1089 us,
+// the two fp64 sums in one instruction to 1068.
 constexpr int kLossWarps = 8;
 
 struct LossArgs {
@@ -139,64 +143,60 @@ __device__ __forceinline__ uint32_t theta_key(const uint32_t (&k)[V], bool valid
     return prefix;
 }
 
-// theta_B from a guess g (the same term's theta at the previous token, which
-// is close: consecutive tokens route alike).  With n = #{k >= g}, theta is
-// the (n - B + 1)-th smallest key >= g, or the (B - n)-th largest key < g;
-// those are taken one distinct value at a time (redux min / max, then the
-// count of that value, so ties count with their multiplicity).  More than
-// kExtract rounds, or a round without a candidate, falls back to the bit
-// search.  Exact either way.
+// A candidate for theta_B from a guess g (the same term's theta at the previous
+// token, which is close: consecutive tokens route alike).  With n = #{k >= g},
+// theta is the (n - B + 1)-th smallest key >= g, or the (B - n)-th largest key
+// < g; those are taken one at a time, as if the keys were distinct (a masked
+// extreme per lane, one redux.sync, and the slots that hold it drop out, on the
+// FMA pipe).  The caller's count proves the result; -1 when it would take more
+// than kExtract rounds.  k: the scores, -1 in idle lanes.
 constexpr int kExtract = 6;
 
-template <int V>
-__device__ __forceinline__ uint32_t theta_near(const uint32_t (&k)[V], bool valid, int top_b,
-                                               uint32_t g) {
-    uint32_t c = 0;
+template <int V, bool ALL_VALID>
+__device__ __forceinline__ float theta_near(const float (&k)[V], int top_b, float g) {
+    float c = kCount0, x[V];
 #pragma unroll
-    for (int j = 0; j < V; ++j) c += valid && k[j] >= g ? 1u : 0u;
-    const int n = (int)__reduce_add_sync(kFull, c);
-    if (n >= top_b) {
-        int r = n - top_b;                          // keys >= g that rank below theta
-        uint32_t lower = g;
-        if (r < kExtract) {
+    for (int j = 0; j < V; ++j) c = __fadd_rn(c, set_ge(k[j], g));
+    const int over = (int)warp_count(c) - top_b;     // keys >= g past theta, from the low end
+    if (over >= 0) {
+        if (over >= kExtract) return -1.f;
+#pragma unroll
+        for (int j = 0; j < V; ++j) x[j] = __fmaf_rn(set_gt(g, k[j]), kFar, k[j]);
+        float mn = warp_min_f(lane_min_f<V>(x));
 #pragma unroll 1
-            for (int it = 0; it < kExtract; ++it) {
-                uint32_t m = 0xffffffffu;
+        for (int i = 0; i < over; ++i) {
 #pragma unroll
-                for (int j = 0; j < V; ++j) m = valid && k[j] >= lower && k[j] < m ? k[j] : m;
-                m = __reduce_min_sync(kFull, m);
-                uint32_t e = 0;
-#pragma unroll
-                for (int j = 0; j < V; ++j) e += valid && k[j] == m ? 1u : 0u;
-                const int ce = (int)__reduce_add_sync(kFull, e);
-                if (ce == 0) break;                 // no key left (m is the sentinel)
-                if (ce > r) return m;
-                r -= ce;
-                lower = m + 1u;
-            }
+            for (int j = 0; j < V; ++j) x[j] = __fmaf_rn(set_eq(x[j], mn), kFar, x[j]);
+            mn = warp_min_f(lane_min_f<V>(x));
         }
-    } else {
-        int need = top_b - n;                       // theta is the need-th largest key < g
-        uint32_t upper = g;
-        if (need <= kExtract) {
-#pragma unroll 1
-            for (int it = 0; it < kExtract; ++it) {
-                uint32_t m = 0u;
-#pragma unroll
-                for (int j = 0; j < V; ++j) m = valid && k[j] < upper && k[j] > m ? k[j] : m;
-                m = __reduce_max_sync(kFull, m);
-                uint32_t e = 0;
-#pragma unroll
-                for (int j = 0; j < V; ++j) e += valid && k[j] < upper && k[j] == m ? 1u : 0u;
-                const int ce = (int)__reduce_add_sync(kFull, e);
-                if (ce == 0) break;                 // no key below `upper`
-                if (ce >= need) return m;
-                need -= ce;
-                upper = m;
-            }
-        }
+        return mn;
     }
-    return theta_key<V>(k, valid, top_b);
+    if (-over > kExtract) return -1.f;
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        x[j] = __fmul_rn(k[j], set_gt(g, k[j]));
+        if (!ALL_VALID) x[j] = fmaxf(x[j], 0.f);     // idle lanes
+    }
+    float mx = warp_max_f(lane_max_f<V>(x));
+#pragma unroll 1
+    for (int i = 1; i < -over; ++i) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) x[j] = __fmaf_rn(-set_eq(x[j], mx), x[j], x[j]);
+        mx = warp_max_f(lane_max_f<V>(x));
+    }
+    return mx;
+}
+
+// Keys above and equal to th, over the warp: above | equal << 10.
+template <int V>
+__device__ __forceinline__ uint32_t theta_counts(const float (&k)[V], float th) {
+    float gt = kCount0, eq = 0.f;
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        gt = __fadd_rn(gt, set_gt(k[j], th));
+        eq = __fadd_rn(eq, set_eq(k[j], th));
+    }
+    return warp_count(__fmaf_rn(eq, 1024.f, gt));
 }
 
 // Slot of this lane holding the element at position B of the total order
@@ -247,17 +247,31 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // w_e = q_e m_e (1 - m_e) = q_e u v, so that dl/ds_e = (W [e = e*] - w_e) / tau
 // with W = sum_e w_e (the second part through theta_B = s_{e*}).  Adds the
 // lane's share of l and of W to loss and wsum; the slot of e* comes back.
-template <int V>
+template <int V, bool ALL_VALID>
 __device__ __forceinline__ int coverage(const float (&s)[V], const float (&q)[V], bool valid,
-                                        int top_b, float k2, int lane, uint32_t& guess,
+                                        int top_b, float k2, int lane, float& guess,
                                         float (&w)[V], float (&om)[V], float& loss, float& wsum) {
-    uint32_t k[V];
+    float k[V];
 #pragma unroll
-    for (int j = 0; j < V; ++j) k[j] = valid ? __float_as_uint(s[j]) : 0u;
-    const uint32_t th = theta_near<V>(k, valid, top_b, guess);
-    guess = th;
-    const int js = theta_slot<V>(k, valid, th, top_b, lane);
-    const float theta = __uint_as_float(th);
+    for (int j = 0; j < V; ++j) k[j] = ALL_VALID || valid ? s[j] : -1.f;
+    float theta = theta_near<V, ALL_VALID>(k, top_b, guess);
+    // theta is the B-th of the order exactly when fewer than B keys are above
+    // it and at least B at or above it
+    uint32_t n = theta >= 0.f ? theta_counts<V>(k, theta) : 1023u;
+    int js = -1;
+    const bool found = (int)(n & 1023u) < top_b && (int)((n & 1023u) + (n >> 10)) >= top_b;
+    if (found && (n >> 10) == 1u) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) js = k[j] == theta ? j : js;
+    } else {
+        uint32_t kb[V];
+#pragma unroll
+        for (int j = 0; j < V; ++j) kb[j] = valid ? __float_as_uint(s[j]) : 0u;
+        const uint32_t th = found ? __float_as_uint(theta) : theta_key<V>(kb, valid, top_b);
+        js = theta_slot<V>(kb, valid, th, top_b, lane);
+        theta = __uint_as_float(th);
+    }
+    guess = theta;
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         const float d = s[j] - theta;
@@ -331,22 +345,22 @@ __device__ __forceinline__ void store_dz3(float* rR, float* rT, float* rS, const
 // Both terms of step t of layer l from s^T = p^R_t + p^T_t, p^S_{rho(t+1,l)}
 // and the target q = p^R_{t+1}: their losses (lane 0: l^T, lane 16: l^ST in
 // the returned value), gT = tau dl^T/ds, gST likewise, and the target parts.
-template <int V>
+template <int V, bool ALL_VALID>
 __device__ __forceinline__ float step_terms(const float (&pR)[V], const float (&pT)[V],
                                             const float (&pS)[V], const float (&q)[V],
                                             bool st, bool valid, int top_b, float k2, int lane,
-                                            uint32_t (&guess)[2], float (&wT)[V], float (&omT)[V],
+                                            float (&guess)[2], float (&wT)[V], float (&omT)[V],
                                             float (&wST)[V], float (&omST)[V]) {
     float s[V];
 #pragma unroll
     for (int j = 0; j < V; ++j) s[j] = __fadd_rn(pR[j], pT[j]);
     float lT = 0.f, sT = 0.f, lST = 0.f, sST = 0.f;
-    const int jT = coverage<V>(s, q, valid, top_b, k2, lane, guess[0], wT, omT, lT, sT);
+    const int jT = coverage<V, ALL_VALID>(s, q, valid, top_b, k2, lane, guess[0], wT, omT, lT, sT);
     int jST = -1;
     if (st) {
 #pragma unroll
         for (int j = 0; j < V; ++j) s[j] = __fadd_rn(s[j], pS[j]);
-        jST = coverage<V>(s, q, valid, top_b, k2, lane, guess[1], wST, omST, lST, sST);
+        jST = coverage<V, ALL_VALID>(s, q, valid, top_b, k2, lane, guess[1], wST, omST, lST, sST);
     }
     const float y = warp_sum4(lT, sT, lST, sST, lane);
     const float WT = __shfl_sync(kFull, y, 8);
@@ -401,8 +415,8 @@ __global__ void __launch_bounds__(32 * kLossWarps, loss_blocks<V>()) cache_loss_
         carry[j] = 0.f;
         wST[j] = omST[j] = pS[j] = 0.f;
     }
-    double sumT = 0.0, sumST = 0.0;
-    uint32_t guess[2] = {0u, 0u};                             // theta^T, theta^ST of the last step
+    double sum = 0.0;
+    float guess[2] = {0.f, 0.f};                              // theta^T, theta^ST of the last step
 
     if (t0 > 0) {
         // halo: the two terms of step t0 - 1 give the target part of p^R_{t0}
@@ -411,7 +425,7 @@ __global__ void __launch_bounds__(32 * kLossWarps, loss_blocks<V>()) cache_loss_
         load_row<V>(pT, hp + N, lane, valid);
         load_row<V>(q, pp, lane, valid);
         if (st) load_row<V>(pS, hp + s_off, lane, valid);
-        step_terms<V>(pR, pT, pS, q, st, valid, a.top_b, k2, lane, guess, wT, omT, wST, omST);
+        step_terms<V, ALL_VALID>(pR, pT, pS, q, st, valid, a.top_b, k2, lane, guess, wT, omT, wST, omST);
 #pragma unroll
         for (int j = 0; j < V; ++j) {
             carry[j] = fmaf(cT, omT[j], cST * omST[j]);
@@ -431,14 +445,12 @@ __global__ void __launch_bounds__(32 * kLossWarps, loss_blocks<V>()) cache_loss_
         if (next) {
             load_row<V>(q, pp + tok, lane, valid);
             if (st) load_row<V>(pS, pp + s_off, lane, valid);
-            const float y = step_terms<V>(pR, pT, pS, q, st, valid, a.top_b, k2, lane, guess, wT,
+            const float y = step_terms<V, ALL_VALID>(pR, pT, pS, q, st, valid, a.top_b, k2, lane, guess, wT,
                                           omT, wST, omST);
-            if (lane == 0) {
-                sumT += (double)y;
-                if (lossp) lossp[0] = y;
-            } else if (lane == 16) {
-                sumST += (double)y;
-                if (lossp) lossp[(size_t)L * 2 + 1] = st ? y : 0.f;
+            // lanes 0 and 16 hold l^T and l^ST, in one fp64 addition
+            if ((lane & 15) == 0) {
+                sum += (double)y;
+                if (lossp) lossp[lane == 0 ? 0 : (size_t)L * 2 + 1] = lane == 0 || st ? y : 0.f;
             }
 #pragma unroll
             for (int j = 0; j < V; ++j) {
@@ -468,8 +480,8 @@ __global__ void __launch_bounds__(32 * kLossWarps, loss_blocks<V>()) cache_loss_
         for (int j = 0; j < V; ++j) pR[j] = q[j];
     }
     if (a.partial) {
-        sumT = __shfl_sync(kFull, sumT, 0);
-        sumST = __shfl_sync(kFull, sumST, 16);
+        const double sumT = __shfl_sync(kFull, sum, 0);
+        const double sumST = __shfl_sync(kFull, sum, 16);
         if (lane == 0) {
             a.partial[(size_t)task * 2 + 0] = sumT;
             a.partial[(size_t)task * 2 + 1] = sumST;
@@ -893,32 +905,49 @@ int launch_loss_rows_kp(LossArgs& a, cudaStream_t stream) {
                         : launch_loss_rows_st<NL, false>(a, stream);
 }
 
-// Means L_T, L_ST: fixed-order sums of the per-task sums (deterministic).
+// Means L_T, L_ST: fixed-order sums of the per-task sums (deterministic).  A
+// cluster of eight CTAs, each summing every eighth round of threads, then added
+// in rank order: an SM adds two doubles a cycle, so one CTA took 25 of its
+// 37 us for the 98,304 additions of 49,152 tasks alone; 12 us with the cluster.
+constexpr int kMeanCtas = 8;
 constexpr int kMeanThreads = 256;
 
 __global__ void __launch_bounds__(kMeanThreads)
-    loss_means_kernel(const double* partial, int tasks, double inv_nT, double inv_nST,
+    loss_means_kernel(const double2* partial, int tasks, double inv_nT, double inv_nST,
                       double* means) {
-    __shared__ double sh[2][kMeanThreads];
-    double aT = 0.0, aST = 0.0;
-    for (int i = threadIdx.x; i < tasks; i += kMeanThreads) {
-        aT += partial[(size_t)i * 2 + 0];
-        aST += partial[(size_t)i * 2 + 1];
+    __shared__ double2 sh[kMeanThreads];
+    const int rank = (int)cluster_ctarank();
+    double2 a = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int i = rank * kMeanThreads + threadIdx.x; i < tasks; i += kMeanCtas * kMeanThreads) {
+        const double2 v = partial[i];
+        a.x += v.x;
+        a.y += v.y;
     }
-    sh[0][threadIdx.x] = aT;
-    sh[1][threadIdx.x] = aST;
+    sh[threadIdx.x] = a;
     __syncthreads();
     for (int w = kMeanThreads / 2; w > 0; w >>= 1) {
         if ((int)threadIdx.x < w) {
-            sh[0][threadIdx.x] += sh[0][threadIdx.x + w];
-            sh[1][threadIdx.x] += sh[1][threadIdx.x + w];
+            sh[threadIdx.x].x += sh[threadIdx.x + w].x;
+            sh[threadIdx.x].y += sh[threadIdx.x + w].y;
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        means[0] = sh[0][0] * inv_nT;
-        means[1] = sh[1][0] * inv_nST;
+    cluster_sync();                          // every CTA's sum is in place
+    if (rank == 0 && threadIdx.x == 0) {
+        double2 t = sh[0];
+        for (uint32_t r = 1; r < (uint32_t)kMeanCtas; ++r) {
+            double2 v;
+            asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];"
+                         : "=d"(v.x), "=d"(v.y)
+                         : "r"(cluster_map(&sh[0], r)));
+            t.x += v.x;
+            t.y += v.y;
+        }
+        means[0] = t.x * inv_nT;
+        means[1] = t.y * inv_nST;
     }
+    cluster_sync();                          // and stays until it has been read
 }
 
 template <int V, bool ALL_VALID>
@@ -1009,12 +1038,25 @@ int launch_cache_loss(const crc_problem& p, const float* probs, int T, int heads
     const double inv_n = n_valid > 0 ? 1.0 / n_valid : 0.0;
     {
         ProfScope prof(CRC_KERNEL_LOSS_MEANS, stream);
-        loss_means_kernel<<<1, kMeanThreads, 0, stream>>>(
-            static_cast<const double*>(workspace), p.B * p.L * a.nchunks, inv_n,
-            heads == 3 ? inv_n : 0.0, means);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kMeanCtas;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t c = {};
+        c.gridDim = dim3(kMeanCtas);
+        c.blockDim = dim3(kMeanThreads);
+        c.stream = stream;
+        c.attrs = at;
+        c.numAttrs = 1;
+        rc = cudaLaunchKernelEx(&c, loss_means_kernel, static_cast<const double2*>(workspace),
+                                p.B * p.L * a.nchunks, inv_n, heads == 3 ? inv_n : 0.0,
+                                means) == cudaSuccess
+                 ? CRC_OK
+                 : CRC_ECUDA;
     }
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return rc;
 }
 
 }  // namespace crc
