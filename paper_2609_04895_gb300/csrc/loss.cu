@@ -909,17 +909,21 @@ int launch_loss_rows_kp(LossArgs& a, cudaStream_t stream) {
 // cluster of eight CTAs, each summing every eighth round of threads, then added
 // in rank order: an SM adds two doubles a cycle, so one CTA took 25 of its
 // 37 us for the 98,304 additions of 49,152 tasks alone; 12 us with the cluster.
+// Few tasks stay on one CTA, which has nothing to exchange: 1024 tasks 3.5 us
+// against 4.5, 2048 4.2 / 4.5, 4096 5.5 / 4.7, 8192 8.1 / 4.9 (launches in a row).
 constexpr int kMeanCtas = 8;
+constexpr int kMeanSmall = 2048;       // tasks that one CTA adds
 constexpr int kMeanThreads = 256;
 
 __global__ void __launch_bounds__(kMeanThreads)
     loss_means_kernel(const double2* partial, int tasks, double inv_nT, double inv_nST,
                       double* means) {
     __shared__ double2 sh[kMeanThreads];
-    const int rank = (int)cluster_ctarank();
+    const int ctas = (int)gridDim.x;         // one cluster
+    const int rank = (int)blockIdx.x;
     double2 a = make_double2(0.0, 0.0);
 #pragma unroll 4
-    for (int i = rank * kMeanThreads + threadIdx.x; i < tasks; i += kMeanCtas * kMeanThreads) {
+    for (int i = rank * kMeanThreads + threadIdx.x; i < tasks; i += ctas * kMeanThreads) {
         const double2 v = partial[i];
         a.x += v.x;
         a.y += v.y;
@@ -933,10 +937,10 @@ __global__ void __launch_bounds__(kMeanThreads)
         }
         __syncthreads();
     }
-    cluster_sync();                          // every CTA's sum is in place
+    if (ctas > 1) cluster_sync();            // every CTA's sum is in place
     if (rank == 0 && threadIdx.x == 0) {
         double2 t = sh[0];
-        for (uint32_t r = 1; r < (uint32_t)kMeanCtas; ++r) {
+        for (uint32_t r = 1; r < (uint32_t)ctas; ++r) {
             double2 v;
             asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];"
                          : "=d"(v.x), "=d"(v.y)
@@ -947,7 +951,7 @@ __global__ void __launch_bounds__(kMeanThreads)
         means[0] = t.x * inv_nT;
         means[1] = t.y * inv_nST;
     }
-    cluster_sync();                          // and stays until it has been read
+    if (ctas > 1) cluster_sync();            // and stays until it has been read
 }
 
 template <int V, bool ALL_VALID>
@@ -1038,20 +1042,21 @@ int launch_cache_loss(const crc_problem& p, const float* probs, int T, int heads
     const double inv_n = n_valid > 0 ? 1.0 / n_valid : 0.0;
     {
         ProfScope prof(CRC_KERNEL_LOSS_MEANS, stream);
+        const int tasks = p.B * p.L * a.nchunks;
+        const int ctas = tasks > kMeanSmall ? kMeanCtas : 1;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = kMeanCtas;
+        at[0].val.clusterDim.x = ctas;
         at[0].val.clusterDim.y = 1;
         at[0].val.clusterDim.z = 1;
         cudaLaunchConfig_t c = {};
-        c.gridDim = dim3(kMeanCtas);
+        c.gridDim = dim3(ctas);
         c.blockDim = dim3(kMeanThreads);
         c.stream = stream;
         c.attrs = at;
-        c.numAttrs = 1;
+        c.numAttrs = ctas > 1 ? 1 : 0;
         rc = cudaLaunchKernelEx(&c, loss_means_kernel, static_cast<const double2*>(workspace),
-                                p.B * p.L * a.nchunks, inv_n, heads == 3 ? inv_n : 0.0,
-                                means) == cudaSuccess
+                                tasks, inv_n, heads == 3 ? inv_n : 0.0, means) == cudaSuccess
                  ? CRC_OK
                  : CRC_ECUDA;
     }
