@@ -66,7 +66,7 @@ cudaEvent_t pool_event() {
         return e;
     }
     cudaEvent_t e = nullptr;
-    if (cudaEventCreate(&e) != cudaSuccess) return nullptr;
+    if (cuda_status(cudaEventCreate(&e))) return nullptr;
     return e;
 }
 
@@ -77,7 +77,7 @@ ProfScope::ProfScope(int kind, cudaStream_t s) : slot(-1), stream(s) {
     if (!g_prof_on || kind < 0 || kind >= CRC_KERNEL_KINDS) return;
     ProfRecord r{kind, pool_event(), pool_event()};
     if (!r.start || !r.stop) return;
-    cudaEventRecord(r.start, s);
+    (void)cuda_status(cudaEventRecord(r.start, s));
     slot = (int)g_prof.size();
     g_prof.push_back(r);
 }
@@ -85,14 +85,14 @@ ProfScope::ProfScope(int kind, cudaStream_t s) : slot(-1), stream(s) {
 ProfScope::~ProfScope() {
     if (slot < 0) return;
     std::lock_guard<std::mutex> lk(g_prof_mu);
-    cudaEventRecord(g_prof[slot].stop, stream);
+    (void)cuda_status(cudaEventRecord(g_prof[slot].stop, stream));
 }
 
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
 uint32_t* device_error_word() {
     void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_device_error) != cudaSuccess) return nullptr;
+    if (cuda_status(cudaGetSymbolAddress(&p, g_device_error))) return nullptr;
     return static_cast<uint32_t*>(p);
 }
 
@@ -137,20 +137,19 @@ int crc_state_read(const crc_problem* p, const void* state_dev, size_t state_byt
     if (rc) return rc;
     if ((rc = check_state(p, state_dev, state_bytes))) return rc;
     if (!out) return CRC_EINVAL;
-    if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess)
-        return CRC_ECUDA;
+    if ((rc = cuda_status(cudaStreamSynchronize(static_cast<cudaStream_t>(stream))))) return rc;
     const StateLayout lay = state_layout(p->B, p->L, p->N);
     const uint8_t* base = static_cast<const uint8_t*>(state_dev);
     StateHeader h;
-    if (cudaMemcpy(&h, base, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return CRC_ECUDA;
+    if ((rc = cuda_status(cudaMemcpy(&h, base, sizeof h, cudaMemcpyDeviceToHost)))) return rc;
     if (h.magic != kStateMagic || h.L != p->L || h.N != p->N || h.K != p->K || h.C != p->C ||
         h.R != p->R || h.B != p->B)
         return CRC_ESTATE;
     const size_t nchains = (size_t)p->B * p->L;
     std::vector<ChainState> ch(nchains);
-    if (cudaMemcpy(ch.data(), base + lay.chains, nchains * sizeof(ChainState),
-                   cudaMemcpyDeviceToHost) != cudaSuccess)
-        return CRC_ECUDA;
+    if ((rc = cuda_status(cudaMemcpy(ch.data(), base + lay.chains, nchains * sizeof(ChainState),
+                                     cudaMemcpyDeviceToHost))))
+        return rc;
     std::memset(out, 0, sizeof *out);
     const int NW = (p->N + 31) / 32;
     for (size_t c = 0; c < nchains; ++c) {
@@ -170,9 +169,9 @@ int crc_state_read(const crc_problem* p, const void* state_dev, size_t state_byt
     out->tokens = (uint64_t)h.t_next;
     out->error = h.error;
     if (retention_host &&
-        cudaMemcpy(retention_host, base + lay.retention, nchains * p->N * sizeof(float),
-                   cudaMemcpyDeviceToHost) != cudaSuccess)
-        return CRC_ECUDA;
+        (rc = cuda_status(cudaMemcpy(retention_host, base + lay.retention,
+                                     nchains * p->N * sizeof(float), cudaMemcpyDeviceToHost))))
+        return rc;
     return h.error ? (int)h.error : CRC_OK;
 }
 
@@ -248,13 +247,12 @@ int crc_state_read_aux(const crc_problem* p, const void* state_dev, size_t state
     if (rc) return rc;
     if ((rc = check_state(p, state_dev, state_bytes))) return rc;
     if (!aux_host) return CRC_EINVAL;
-    if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess) return CRC_ECUDA;
+    if ((rc = cuda_status(cudaStreamSynchronize(static_cast<cudaStream_t>(stream))))) return rc;
     const StateLayout lay = state_layout(p->B, p->L, p->N);
     const uint8_t* base = static_cast<const uint8_t*>(state_dev);
-    if (cudaMemcpy(aux_host, base + lay.aux, (size_t)p->B * p->L * p->N * sizeof(uint32_t),
-                   cudaMemcpyDeviceToHost) != cudaSuccess)
-        return CRC_ECUDA;
-    return CRC_OK;
+    return cuda_status(cudaMemcpy(aux_host, base + lay.aux,
+                                  (size_t)p->B * p->L * p->N * sizeof(uint32_t),
+                                  cudaMemcpyDeviceToHost));
 }
 
 size_t crc_fused_workspace_bytes(const crc_problem* p) {
@@ -345,42 +343,40 @@ int crc_route_and_cache_host(const crc_problem* p, const uint16_t* hidden_host,
     cudaStream_t cs = nullptr;
     cudaEvent_t entry = nullptr, joined = nullptr, copied[2] = {nullptr, nullptr},
                 done[2] = {nullptr, nullptr};
-    bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
+    rc = cuda_status(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     for (cudaEvent_t* e : {&entry, &joined, &copied[0], &copied[1], &done[0], &done[1]})
-        ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+        if (rc == CRC_OK) rc = cuda_status(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     // the staging halves may still be read by work queued earlier on `stream`
-    ok = ok && cudaEventRecord(entry, s) == cudaSuccess &&
-         cudaStreamWaitEvent(cs, entry, 0) == cudaSuccess;
-    rc = ok ? CRC_OK : CRC_ECUDA;
+    if (rc == CRC_OK) rc = cuda_status(cudaEventRecord(entry, s));
+    if (rc == CRC_OK) rc = cuda_status(cudaStreamWaitEvent(cs, entry, 0));
     for (int t0 = 0, i = 0; rc == CRC_OK && t0 < T; t0 += chunk, ++i) {
         const int n = (T - t0) < chunk ? (T - t0) : chunk;
         const int j = i & 1;
         uint8_t* buf = static_cast<uint8_t*>(staging_dev) + (size_t)j * half;
         const uint8_t* src = reinterpret_cast<const uint8_t*>(hidden_host) + (size_t)t0 * row;
-        if (i >= 2 && cudaStreamWaitEvent(cs, done[j], 0) != cudaSuccess) rc = CRC_ECUDA;
+        if (i >= 2) rc = cuda_status(cudaStreamWaitEvent(cs, done[j], 0));
         // [B][n][L][d] of the chunk, stream b's tokens at pitch T * row in host memory
         if (rc == CRC_OK && two_d) {
-            if (cudaMemcpy2DAsync(buf, (size_t)n * row, src, (size_t)T * row, (size_t)n * row,
-                                  (size_t)p->B, cudaMemcpyHostToDevice, cs) != cudaSuccess)
-                rc = CRC_ECUDA;
+            rc = cuda_status(cudaMemcpy2DAsync(buf, (size_t)n * row, src, (size_t)T * row,
+                                               (size_t)n * row, (size_t)p->B,
+                                               cudaMemcpyHostToDevice, cs));
         } else {
             for (int b = 0; rc == CRC_OK && b < p->B; ++b)
-                if (cudaMemcpyAsync(buf + (size_t)b * n * row, src + (size_t)b * T * row,
-                                    (size_t)n * row, cudaMemcpyHostToDevice, cs) != cudaSuccess)
-                    rc = CRC_ECUDA;
+                rc = cuda_status(cudaMemcpyAsync(buf + (size_t)b * n * row,
+                                                 src + (size_t)b * T * row, (size_t)n * row,
+                                                 cudaMemcpyHostToDevice, cs));
         }
-        if (rc == CRC_OK && (cudaEventRecord(copied[j], cs) != cudaSuccess ||
-                             cudaStreamWaitEvent(s, copied[j], 0) != cudaSuccess))
-            rc = CRC_ECUDA;
+        if (rc == CRC_OK) rc = cuda_status(cudaEventRecord(copied[j], cs));
+        if (rc == CRC_OK) rc = cuda_status(cudaStreamWaitEvent(s, copied[j], 0));
         if (rc == CRC_OK)
             rc = crc_route_and_cache(p, reinterpret_cast<const uint16_t*>(buf), w_cat_dev, n,
                                      state_dev, state_bytes, nullptr, workspace_dev,
                                      workspace_bytes, stream);
-        if (rc == CRC_OK && cudaEventRecord(done[j], s) != cudaSuccess) rc = CRC_ECUDA;
+        if (rc == CRC_OK) rc = cuda_status(cudaEventRecord(done[j], s));
     }
     // everything the call queued on its copy stream is ordered before later work on `stream`
-    if (cs && joined && cudaEventRecord(joined, cs) == cudaSuccess)
-        cudaStreamWaitEvent(s, joined, 0);
+    if (cs && joined && cuda_status(cudaEventRecord(joined, cs)) == CRC_OK)
+        (void)cuda_status(cudaStreamWaitEvent(s, joined, 0));
     for (cudaEvent_t e : {entry, joined, copied[0], copied[1], done[0], done[1]})
         if (e) cudaEventDestroy(e);
     if (cs) cudaStreamDestroy(cs);
@@ -426,10 +422,9 @@ int crc_host_alloc(size_t bytes, void** out) {
     madvise(p, body, MADV_HUGEPAGE);    // advisory: base pages if huge pages are unavailable
 #endif
     for (size_t o = 0; o < body; o += hp) p[o] = 0;
-    if (cudaHostRegister(p, body, cudaHostRegisterDefault) != cudaSuccess) {
-        cudaGetLastError();
+    if (const int rc = cuda_status(cudaHostRegister(p, body, cudaHostRegisterDefault))) {
         munmap(base, len);
-        return CRC_ECUDA;
+        return rc;
     }
     {
         std::lock_guard<std::mutex> lk(g_host_mu);
@@ -449,7 +444,7 @@ int crc_host_free(void* ptr) {
         m = it->second;
         g_host_maps.erase(it);
     }
-    const int rc = cudaHostUnregister(ptr) == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    const int rc = cuda_status(cudaHostUnregister(ptr));
     munmap(m.base, m.len);
     return rc;
 }
@@ -486,10 +481,11 @@ int crc_cache_loss(const crc_problem* p, const float* probs_dev, int32_t T, int3
 }
 
 int crc_device_error(void) {
-    if (cudaDeviceSynchronize() != cudaSuccess) return CRC_ECUDA;
+    int rc = cuda_status(cudaDeviceSynchronize());
     uint32_t v = 0, zero = 0;
-    if (cudaMemcpyFromSymbol(&v, g_device_error, sizeof v) != cudaSuccess) return CRC_ECUDA;
-    if (cudaMemcpyToSymbol(g_device_error, &zero, sizeof zero) != cudaSuccess) return CRC_ECUDA;
+    if (rc == CRC_OK) rc = cuda_status(cudaMemcpyFromSymbol(&v, g_device_error, sizeof v));
+    if (rc == CRC_OK) rc = cuda_status(cudaMemcpyToSymbol(g_device_error, &zero, sizeof zero));
+    if (rc != CRC_OK) return rc;
     return (int)v;
 }
 
@@ -513,8 +509,8 @@ int crc_profile_end(crc_kernel_times* out) {
     int rc = CRC_OK;
     for (auto& r : g_prof) {
         float ms = 0.f;
-        if (cudaEventSynchronize(r.stop) != cudaSuccess ||
-            cudaEventElapsedTime(&ms, r.start, r.stop) != cudaSuccess) {
+        if (cuda_status(cudaEventSynchronize(r.stop)) ||
+            cuda_status(cudaEventElapsedTime(&ms, r.start, r.stop))) {
             rc = CRC_ECUDA;
             continue;
         }

@@ -9,6 +9,15 @@
 
 namespace crc {
 
+// The code of a runtime call's result.  A refused call also leaves its error as
+// the thread's last one, where the next launch that asks for it would take it
+// for its own: it is cleared here.
+inline int cuda_status(cudaError_t e) {
+    if (e == cudaSuccess) return CRC_OK;
+    (void)cudaGetLastError();
+    return CRC_ECUDA;
+}
+
 // Count of kernels launched by the library (reported by crc_launch_count).
 void note_launch();
 

@@ -147,7 +147,7 @@ int launch_fused_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
     if (!make_hidden_map(&mh, hidden, p.B, T, p.L, p.d, f.TB, f.SB)) return CRC_ECUDA;
     if (!make_weight_map(&mw, w_cat, p.L, 3 * NH, p.d, Cfg::B_BOX_ROWS)) return CRC_ECUDA;
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    if (cudaMemsetAsync(ws, 0, f.ctl_bytes, stream) != cudaSuccess) return CRC_ECUDA;
+    if (const int rc = cuda_status(cudaMemsetAsync(ws, 0, f.ctl_bytes, stream))) return rc;
     FusedArgs a;
     a.state = static_cast<uint8_t*>(state);
     a.B = p.B;
@@ -215,7 +215,7 @@ int launch_fused_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
                                         Cfg::SMEM_BYTES, stream);
     }
     note_launch();
-    return e == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(e);
 }
 
 // The GEMM on CTA pairs (N = 128: three heads, or two in update-only mode)

@@ -868,9 +868,9 @@ int launch_loss_rows(LossArgs& a, cudaStream_t stream) {
     static std::atomic<int> blocks_per_sm{0};
     if (blocks_per_sm.load() == 0) {
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cache_loss_rows_kernel<NL, KP, ST>,
-                                                          32 * kRowWarps, 0) != cudaSuccess)
-            return CRC_ECUDA;
+        const int rc = cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &n, cache_loss_rows_kernel<NL, KP, ST>, 32 * kRowWarps, 0));
+        if (rc) return rc;
         blocks_per_sm.store(n > 0 ? n : 1);
     }
     const long long groups = (a.B * (long long)a.L + CPW - 1) / CPW;
@@ -888,7 +888,7 @@ int launch_loss_rows(LossArgs& a, cudaStream_t stream) {
         cache_loss_rows_kernel<NL, KP, ST><<<grid, 32 * kRowWarps, 0, stream>>>(a);
     }
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(cudaGetLastError());
 }
 
 template <int NL, bool ST>
@@ -966,7 +966,7 @@ int launch_loss_t(const LossArgs& a, cudaStream_t stream) {
             cache_loss_kernel<V, ALL_VALID, false><<<grid, 32 * kLossWarps, 0, stream>>>(a);
     }
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(cudaGetLastError());
 }
 
 }  // namespace
@@ -1055,10 +1055,9 @@ int launch_cache_loss(const crc_problem& p, const float* probs, int T, int heads
         c.stream = stream;
         c.attrs = at;
         c.numAttrs = ctas > 1 ? 1 : 0;
-        rc = cudaLaunchKernelEx(&c, loss_means_kernel, static_cast<const double2*>(workspace),
-                                tasks, inv_n, heads == 3 ? inv_n : 0.0, means) == cudaSuccess
-                 ? CRC_OK
-                 : CRC_ECUDA;
+        rc = cuda_status(cudaLaunchKernelEx(&c, loss_means_kernel,
+                                            static_cast<const double2*>(workspace), tasks, inv_n,
+                                            heads == 3 ? inv_n : 0.0, means));
     }
     note_launch();
     return rc;

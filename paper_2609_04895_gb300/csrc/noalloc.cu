@@ -22,12 +22,12 @@ std::vector<void*> g_scratch_ptr;   // device address of the array, per device
 // would leave it stale, which is why the entry point does not support one.
 int scratch_for_current_device(void** out) {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return CRC_ECUDA;
+    if (const int rc = crc::cuda_status(cudaGetDevice(&dev))) return rc;
     std::lock_guard<std::mutex> lk(g_scratch_mu);
     if ((int)g_scratch_ptr.size() <= dev) g_scratch_ptr.resize(dev + 1, nullptr);
     if (!g_scratch_ptr[dev]) {
         void* p = nullptr;
-        if (cudaGetSymbolAddress((void**)&p, g_noalloc_scratch) != cudaSuccess || !p)
+        if (crc::cuda_status(cudaGetSymbolAddress((void**)&p, g_noalloc_scratch)) || !p)
             return CRC_ECUDA;
         g_scratch_ptr[dev] = p;
     }

@@ -42,7 +42,7 @@ int launch_policy_t(const crc_problem& p, const float* scores, int T, void* stat
             <<<grid, 32 * warps_per_block, 0, stream>>>(a);
     }
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(cudaGetLastError());
 }
 
 template <int POL>

@@ -41,10 +41,10 @@ extern "C" int crc_wait_probe(const crc_problem* p, void* state_dev, size_t stat
     if (limit_ns > kWaitLimitNs) limit_ns = kWaitLimitNs;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     void* words = nullptr;
-    if (cudaGetSymbolAddress(&words, g_probe_words) != cudaSuccess) return CRC_ECUDA;
-    if (cudaMemsetAsync(words, 0, sizeof(g_probe_words), s) != cudaSuccess) return CRC_ECUDA;
+    if (const int rc = cuda_status(cudaGetSymbolAddress(&words, g_probe_words))) return rc;
+    if (const int rc = cuda_status(cudaMemsetAsync(words, 0, sizeof(g_probe_words), s))) return rc;
     uint32_t* err = &static_cast<StateHeader*>(state_dev)->error;
     wait_probe_kernel<<<1, 32, 0, s>>>(err, kind, limit_ns);
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(cudaGetLastError());
 }

@@ -123,7 +123,7 @@ int launch_router_pair(const crc_problem& p, const uint16_t* w_cat, const CUtens
         e = cudaLaunchKernelExC(&c, (const void*)kern, args);
     }
     note_launch();
-    return e == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(e);
 }
 
 template <int NH, int H>
@@ -158,10 +158,10 @@ int launch_router_t(const crc_problem& p, const uint16_t* hidden, int T_total, i
     a.kblocks = (p.d + Cfg::BK - 1) / Cfg::BK;
     static bool attr_set = false;   // per instantiation
     if (!attr_set) {
-        if (cudaFuncSetAttribute(router_heads_kernel<NH, H>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 Cfg::SMEM_BYTES) != cudaSuccess)
-            return CRC_ECUDA;
+        const int rc = cuda_status(cudaFuncSetAttribute(
+            router_heads_kernel<NH, H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            Cfg::SMEM_BYTES));
+        if (rc) return rc;
         attr_set = true;
     }
     if constexpr (NH == 128) {
@@ -174,7 +174,7 @@ int launch_router_t(const crc_problem& p, const uint16_t* hidden, int T_total, i
         router_heads_kernel<NH, H><<<grid, Cfg::THREADS, Cfg::SMEM_BYTES, stream>>>(mh, mw, ms, a);
     }
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(cudaGetLastError());
 }
 
 }  // namespace

@@ -21,13 +21,13 @@ __global__ void state_init_kernel(uint8_t* state, crc_problem p) {
 }  // namespace
 
 int launch_state_init(const crc_problem& p, void* state, size_t bytes, cudaStream_t stream) {
-    if (cudaMemsetAsync(state, 0, bytes, stream) != cudaSuccess) return CRC_ECUDA;
+    if (const int rc = cuda_status(cudaMemsetAsync(state, 0, bytes, stream))) return rc;
     {
         ProfScope prof(CRC_KERNEL_STATE, stream);
         state_init_kernel<<<1, 1, 0, stream>>>(static_cast<uint8_t*>(state), p);
     }
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(cudaGetLastError());
 }
 
 template int launch_scan_mode<false>(const crc_problem&, const float*, int, void*,

@@ -37,7 +37,7 @@ int launch_scan_t(const crc_problem& p, const float* scores, int T, void* state,
         cache_scan_kernel<V, ALL_VALID, KP, TRACED><<<grid, 32 * warps_per_block, 0, stream>>>(a);
     }
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(cudaGetLastError());
 }
 
 template <bool TRACED>

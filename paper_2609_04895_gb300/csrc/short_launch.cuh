@@ -72,11 +72,9 @@ int launch_short_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
     cudaGetDevice(&dev);
     const uint64_t bit = dev < 64 ? 1ull << dev : 0;
     if (bit == 0 || !(ready.load() & bit)) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kShortSmem2) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return CRC_ECUDA;
-        }
+        const int rc = cuda_status(cudaFuncSetAttribute(
+            kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kShortSmem2));
+        if (rc) return rc;
         ready.fetch_or(bit);
     }
     cudaLaunchAttribute at[1];
@@ -98,7 +96,7 @@ int launch_short_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
         e = cudaLaunchKernelExC(&c, (const void*)kern, args);
     }
     note_launch();
-    return e == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(e);
 }
 
 template <int NH, int V, bool ALL_VALID>

@@ -157,15 +157,15 @@ int launch_synth_hidden(int B, int T, int L, int d, int t0, uint32_t seed, doubl
     const int blocks = B * ((d / 2 + kSynthPairs - 1) / kSynthPairs);
     const size_t smem = (size_t)L * kSynthPairs * sizeof(float2);
     if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(synth_hidden_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
+        cuda_status(cudaFuncSetAttribute(synth_hidden_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
         return CRC_EUNSUPPORTED;
     {
         ProfScope prof(CRC_KERNEL_SYNTH, stream);
         synth_hidden_kernel<<<blocks, kSynthPairs, smem, stream>>>(a);
     }
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(cudaGetLastError());
 }
 
 int launch_synth_weights(int L, int N, int d, uint32_t seed, int copy_init, uint16_t* out,
@@ -185,7 +185,7 @@ int launch_synth_weights(int L, int N, int d, uint32_t seed, int copy_init, uint
         synth_weights_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0, stream>>>(a);
     }
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? CRC_OK : CRC_ECUDA;
+    return cuda_status(cudaGetLastError());
 }
 
 }  // namespace crc

@@ -138,9 +138,10 @@ int crc_transfer_replay(const crc_problem* p, const crc_transfer* plan, int64_t 
     for (int64_t i = 0; i < n; ++i) {
         const crc_transfer& x = plan[i];
         const int64_t src = ((int64_t)x.l * N + x.expert) % pool_experts;
-        if (cudaMemcpyAsync(slots + ((size_t)x.l * C + x.slot) * eb, pool + (size_t)src * eb, eb,
-                            cudaMemcpyHostToDevice, s) != cudaSuccess)
-            return CRC_ECUDA;
+        if (const int rc = cuda_status(
+                cudaMemcpyAsync(slots + ((size_t)x.l * C + x.slot) * eb, pool + (size_t)src * eb,
+                                eb, cudaMemcpyHostToDevice, s)))
+            return rc;
     }
     return CRC_OK;
 }
