@@ -233,15 +233,14 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
             up += tok;
         };
         float theta = 0.f, th = 0.f;             // Top-K thresholds: lane j token t + j's; t's
+        auto thresholds = [&](int t) {           // (a rank-order trace needs none)
+            if (t + lane < T) theta = row_theta_k<KP>(row0 + (size_t)(t + lane) * tok, N, a.K);
+            th = __shfl_sync(kFull, theta, 0);
+        };
         auto step = [&](int t) {
             float pR[V], pS[V];
             ring_read<V>(&mine[t % D][0][lane * V], pR);
             ring_read<V>(&mine[t % D][ROWS - 1][lane * V], pS);
-            if ((t & 31) == 0) {
-                if (t + lane < T)
-                    theta = row_theta_k<KP>(row0 + (size_t)(t + lane) * tok, N, a.K);
-                th = __shfl_sync(kFull, theta, 0);
-            }
             Sel<V> s;
             const size_t unit = ((size_t)b * a.trace_T + a.trace_t0 + t) * L + l;
             if (rank_order)
@@ -260,6 +259,7 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
 #pragma unroll 1
         for (int t = 0; t < T; ++t) {
             load(t + D - 1);
+            if (!rank_order && (t & 31) == 0) thresholds(t);
             ring_wait<D - 1>();                  // token t's copies have landed
             step(t);
             th = __shfl_sync(kFull, theta, (t + 1) & 31);

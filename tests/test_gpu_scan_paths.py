@@ -2,7 +2,8 @@
 the oracle's literal scans: scores that tie at the Top-K threshold, in the
 refinement and in the evictions (the general forms), scores far above
 probabilities, and comparison-policy states whose token counter has passed the
-range in which priority and expert index share a word.
+range in which priority and expert index share a word.  What those paths may
+cost next to the ordinary ones is bounded too, with wide margins.
 """
 import numpy as np
 import pytest
@@ -68,3 +69,30 @@ def test_policy_priorities_past_the_packed_range(C, policy, N, K, C_):
                     tr.proactive.cpu().numpy()))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+def scan_ms(C, p, x, policy, trace):
+    """Device time of one scan, the least of five."""
+    st = C.State(p)
+    best = 1e9
+    for _ in range(5):
+        st.init()
+        C.crc_profile_begin()
+        if policy == "method":
+            C.cache_scan(p, x, st, trace)
+        else:
+            C.cache_scan_policy(p, x, st, policy, trace)
+        best = min(best, C.crc_profile_end()["scan"]["ms"])
+    return best
+
+
+@pytest.mark.parametrize("policy", ["method", "lru"])
+def test_rank_order_takes_no_thresholds(C, policy):
+    """A rank-order trace takes the whole order and has no use for the Top-K
+    thresholds, which are most of a one-token scan for K = 32: with it the scan is
+    the shorter one (half of it; longer by a quarter when both were taken)."""
+    w = S.TINY.with_(N=128, K=32, C=64, R=4, B=64, T=1, L=24)
+    p = C.problem_of(w)
+    x = torch.from_numpy(scores(w, 5, 1 << 20)).cuda()
+    ranked = scan_ms(C, p, x, policy, C.Trace.alloc(p, w.T))
+    assert ranked < 0.85 * scan_ms(C, p, x, policy, None)
