@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
                 sel_above<V, ALL_VALID>(pR, th, valid, s);
             policy_step<V, ALL_VALID, POL>(
                 cr, aux, pR, pS, want_s && t0 + t >= 1, valid, lane, pa, (uint32_t)(t0 + t),
-                s, [&](Sel<V>& x) { sel_ties<V>(pR, valid, lane, a.K, x); },
+                s, [&](Sel<V>& x) { sel_ties<V>(pR, th, valid, lane, a.K, x); },
                 a.trace_miss ? a.trace_miss + unit : nullptr,
                 a.trace_pro ? a.trace_pro + unit : nullptr);
         };

@@ -71,6 +71,31 @@ def test_policy_priorities_past_the_packed_range(C, policy, N, K, C_):
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("policy", ["method", "lru", "spatio_lru"])
+@pytest.mark.parametrize("N,K,C_,R", [(32, 4, 8, 2), (64, 6, 16, 3), (128, 8, 32, 4),
+                                      (256, 32, 40, 6)])
+def test_rows_no_threshold_settles(C, policy, N, K, C_, R):
+    """Rows of NaN (hidden states that overflowed) have no threshold: the untraced
+    scan takes the same set for them as the ranked one, and goes on as it does."""
+    w = S.TINY.with_(N=N, K=K, C=C_, R=R, B=2, T=40, L=3)
+    x = scores(w, 5, 1 << 16)
+    x[:, 7] = np.nan
+    x[1, 33, 1] = np.nan
+    x = torch.from_numpy(x).cuda()
+    p = C.problem_of(w)
+    got = []
+    for tr in (None, C.Trace.alloc(p, w.T)):
+        st = C.State(p)
+        if policy == "method":
+            C.cache_scan(p, x, st, tr)
+        else:
+            C.cache_scan_policy(p, x, st, policy, tr)
+        g = st.read(want_caches=True, want_chain_counters=True)
+        got.append((g["cache_bits"], g["chain_counters"]))
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
+
+
 def scan_ms(C, p, x, policy, trace):
     """Device time of one scan, the least of five."""
     st = C.State(p)
@@ -96,3 +121,14 @@ def test_rank_order_takes_no_thresholds(C, policy):
     x = torch.from_numpy(scores(w, 5, 1 << 20)).cuda()
     ranked = scan_ms(C, p, x, policy, C.Trace.alloc(p, w.T))
     assert ranked < 0.85 * scan_ms(C, p, x, policy, None)
+
+
+@pytest.mark.parametrize("policy", ["lru", "lfu"])
+def test_tied_rows_cost_about_the_same(C, policy):
+    """Rows whose scores tie at the threshold are settled without K pops over the
+    warp: about 1.35 of the untied rows' time (4.8 with the pops)."""
+    w = S.TINY.with_(N=128, K=32, C=64, R=4, B=1, T=300, L=24)
+    p = C.problem_of(w)
+    tied = torch.from_numpy(scores(w, 5, 8)).cuda()
+    untied = torch.from_numpy(scores(w, 5, 1 << 20)).cuda()
+    assert scan_ms(C, p, tied, policy, None) < 2.5 * scan_ms(C, p, untied, policy, None)
