@@ -187,6 +187,49 @@ __device__ __forceinline__ float theta_near(const float (&k)[V], int top_b, floa
     return mx;
 }
 
+// theta_B from the guess when keys tie: the same walk one distinct value at a
+// time, each with its multiplicity (a count a round), else the bit search.  Bit
+// 31 of the result, which no key has, says that ties were met.
+template <int V>
+struct LossKeys {
+    uint32_t k[V];
+};
+template <int V>
+__device__ __noinline__ uint32_t theta_walk(LossKeys<V> key, bool valid, int top_b, uint32_t g) {
+    constexpr uint32_t kTies = 0x80000000u;
+    const uint32_t (&k)[V] = key.k;
+    uint32_t c = 0;
+#pragma unroll
+    for (int j = 0; j < V; ++j) c += valid && k[j] >= g ? 1u : 0u;
+    int left = (int)__reduce_add_sync(kFull, c) - top_b;     // as `over` in theta_near
+    const bool up = left >= 0;
+    if (!up) left = -left - 1;
+    uint32_t at = g, ties = 0u;              // the walk has taken the keys from g up to (down to) at
+    if (left < kExtract) {
+#pragma unroll 1
+        for (int it = 0; it < kExtract; ++it) {
+            uint32_t m = up ? 0xffffffffu : 0u, e = 0;
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                if (up)
+                    m = valid && k[j] >= at && k[j] < m ? k[j] : m;
+                else
+                    m = valid && k[j] < at && k[j] > m ? k[j] : m;
+            }
+            m = up ? __reduce_min_sync(kFull, m) : __reduce_max_sync(kFull, m);
+#pragma unroll
+            for (int j = 0; j < V; ++j) e += valid && (up || k[j] < at) && k[j] == m ? 1u : 0u;
+            const int n = (int)__reduce_add_sync(kFull, e);
+            if (n == 0) break;               // no key left that way
+            if (n > 1) ties = kTies;
+            if (n > left) return m | ties;
+            left -= n;
+            at = up ? m + 1u : m;
+        }
+    }
+    return theta_key<V>(k, valid, top_b) | ties;
+}
+
 // Keys above and equal to th, over the warp: above | equal << 10.
 template <int V>
 __device__ __forceinline__ uint32_t theta_counts(const float (&k)[V], float th) {
@@ -247,6 +290,9 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // w_e = q_e m_e (1 - m_e) = q_e u v, so that dl/ds_e = (W [e = e*] - w_e) / tau
 // with W = sum_e w_e (the second part through theta_B = s_{e*}).  Adds the
 // lane's share of l and of W to loss and wsum; the slot of e* comes back.
+// guess holds theta of the previous token, negated when keys tied near it: such
+// rows go to theta_walk at once (64 x 200 tokens, N = 128, B = 20, rows on a grid
+// of 1/512: 665 us, and 1047 with theta_near and the bit search for each row).
 template <int V, bool ALL_VALID>
 __device__ __forceinline__ int coverage(const float (&s)[V], const float (&q)[V], bool valid,
                                         int top_b, float k2, int lane, float& guess,
@@ -254,24 +300,32 @@ __device__ __forceinline__ int coverage(const float (&s)[V], const float (&q)[V]
     float k[V];
 #pragma unroll
     for (int j = 0; j < V; ++j) k[j] = ALL_VALID || valid ? s[j] : -1.f;
-    float theta = theta_near<V, ALL_VALID>(k, top_b, guess);
+    const bool tied = signbit(guess);            // keys tied near theta at the previous token
+    float theta = tied ? -1.f : theta_near<V, ALL_VALID>(k, top_b, guess);
     // theta is the B-th of the order exactly when fewer than B keys are above
     // it and at least B at or above it
     uint32_t n = theta >= 0.f ? theta_counts<V>(k, theta) : 1023u;
     int js = -1;
+    uint32_t ties = 0u;
     const bool found = (int)(n & 1023u) < top_b && (int)((n & 1023u) + (n >> 10)) >= top_b;
     if (found && (n >> 10) == 1u) {
 #pragma unroll
         for (int j = 0; j < V; ++j) js = k[j] == theta ? j : js;
     } else {
-        uint32_t kb[V];
+        LossKeys<V> kb;
 #pragma unroll
-        for (int j = 0; j < V; ++j) kb[j] = valid ? __float_as_uint(s[j]) : 0u;
-        const uint32_t th = found ? __float_as_uint(theta) : theta_key<V>(kb, valid, top_b);
-        js = theta_slot<V>(kb, valid, th, top_b, lane);
+        for (int j = 0; j < V; ++j) kb.k[j] = valid ? __float_as_uint(s[j]) : 0u;
+        uint32_t th = __float_as_uint(theta);
+        if (!found)
+            th = tied || theta >= 0.f
+                     ? theta_walk<V>(kb, valid, top_b, __float_as_uint(fabsf(guess)))
+                     : theta_key<V>(kb.k, valid, top_b);
+        ties = th & 0x80000000u;
+        th &= 0x7fffffffu;
+        js = theta_slot<V>(kb.k, valid, th, top_b, lane);
         theta = __uint_as_float(th);
     }
-    guess = theta;
+    guess = __uint_as_float(__float_as_uint(theta) | ties);
 #pragma unroll
     for (int j = 0; j < V; ++j) {
         const float d = s[j] - theta;
