@@ -96,19 +96,21 @@ uint32_t* device_error_word() {
     return static_cast<uint32_t*>(p);
 }
 
-int sm_count() {
+int current_device() {
     int dev = 0;
-    cudaGetDevice(&dev);
-    static std::mutex mu;
-    static std::vector<int> cache;
-    std::lock_guard<std::mutex> lk(mu);
-    if ((int)cache.size() <= dev) cache.resize(dev + 1, 0);
-    if (cache[dev] == 0) {
-        int n = 0;
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        cache[dev] = n > 0 ? n : 1;
-    }
-    return cache[dev];
+    (void)cuda_status(cudaGetDevice(&dev));
+    return dev;
+}
+
+int sm_count() {
+    static PerDevice sms;
+    const int dev = current_device();
+    const int n = sms.get(dev, [&] {
+        int v = 0;
+        (void)cuda_status(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
+        return v;
+    });
+    return n > 0 ? n : 1;
 }
 
 }  // namespace crc

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/crc.h"
+#include "per_device.h"
 
 namespace crc {
 
@@ -33,7 +34,8 @@ struct ProfScope {
 // Library-wide device error word for calls without a state.
 uint32_t* device_error_word();
 
-// Streaming multiprocessors of the current device.
+// The current device and its streaming multiprocessors.
+int current_device();
 int sm_count();
 
 // Router heads over tokens [t_begin, t_begin + T_ext) of hidden [B][T_total][L][d];

@@ -101,16 +101,12 @@ int launch_fused_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
     const FusedPlan f = fused_plan(p, T);
     if (PAIR && f.n_bg % 2 != 0) return CRC_EUNSUPPORTED;
     auto kern = fused_route_cache_kernel<NH, H, V, ALL_VALID, KP, PAIR, TRACED>;
-    // -1: not set up yet in this process; 0: refused; else the grid
-    static int grid = -1;
-    if (grid == 0) return CRC_EUNSUPPORTED;
-    if (grid < 0) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 Cfg::SMEM_BYTES) != cudaSuccess) {
-            (void)cudaGetLastError();
-            grid = 0;
-            return CRC_EUNSUPPORTED;
-        }
+    static PerDevice grids;                    // CTAs of the launch; -1: the device refuses it
+    const int dev = current_device();
+    const int grid = grids.get(dev, [&] {
+        if (cuda_status(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             Cfg::SMEM_BYTES)))
+            return 0;
         if (PAIR) {
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
@@ -124,25 +120,16 @@ int launch_fused_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
             c.attrs = at;
             c.numAttrs = 1;
             int ncl = 0;
-            if (cudaOccupancyMaxActiveClusters(&ncl, (const void*)kern, &c) != cudaSuccess ||
-                ncl < 1) {
-                (void)cudaGetLastError();
-                grid = 0;
-                return CRC_EUNSUPPORTED;
-            }
-            grid = std::min(2 * ncl, sm_count() / 2 * 2);
-        } else {
-            int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, Cfg::MAX_THREADS,
-                                                              Cfg::SMEM_BYTES) != cudaSuccess ||
-                per_sm < 1) {
-                (void)cudaGetLastError();
-                grid = 0;
-                return CRC_EUNSUPPORTED;
-            }
-            grid = sm_count();
+            if (cuda_status(cudaOccupancyMaxActiveClusters(&ncl, (const void*)kern, &c))) return 0;
+            return ncl > 0 ? std::min(2 * ncl, sm_count() / 2 * 2) : -1;
         }
-    }
+        int per_sm = 0;
+        if (cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &per_sm, kern, Cfg::MAX_THREADS, Cfg::SMEM_BYTES)))
+            return 0;
+        return per_sm > 0 ? sm_count() : -1;
+    });
+    if (grid < 1) return CRC_EUNSUPPORTED;
     CUtensorMap mh, mw;
     if (!make_hidden_map(&mh, hidden, p.B, T, p.L, p.d, f.TB, f.SB)) return CRC_ECUDA;
     if (!make_weight_map(&mw, w_cat, p.L, 3 * NH, p.d, Cfg::B_BOX_ROWS)) return CRC_ECUDA;
@@ -204,9 +191,8 @@ int launch_fused_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
             ProfScope prof(CRC_KERNEL_FUSED, stream);
             e = cudaLaunchKernelExC(&c, (const void*)kern, args);
         }
-        if (e != cudaSuccess) {
-            (void)cudaGetLastError();
-            grid = 0;
+        if (cuda_status(e)) {
+            grids.set(dev, -1);
             return CRC_EUNSUPPORTED;
         }
     } else {

@@ -35,8 +35,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
-
 #include "cache_scan.cuh"
 #include "crc_internal.h"
 
@@ -919,16 +917,17 @@ __global__ void __launch_bounds__(32 * kRowWarps, 3) cache_loss_rows_kernel(cons
 template <int NL, int KP, bool ST>
 int launch_loss_rows(LossArgs& a, cudaStream_t stream) {
     constexpr int CPW = 32 / NL;
-    static std::atomic<int> blocks_per_sm{0};
-    if (blocks_per_sm.load() == 0) {
+    static PerDevice resident_blocks;
+    const int blocks_per_sm = resident_blocks.get(current_device(), [] {
         int n = 0;
-        const int rc = cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &n, cache_loss_rows_kernel<NL, KP, ST>, 32 * kRowWarps, 0));
-        if (rc) return rc;
-        blocks_per_sm.store(n > 0 ? n : 1);
-    }
+        if (cuda_status(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &n, cache_loss_rows_kernel<NL, KP, ST>, 32 * kRowWarps, 0)))
+            return 0;
+        return n > 0 ? n : 1;
+    });
+    if (blocks_per_sm < 1) return CRC_ECUDA;
     const long long groups = (a.B * (long long)a.L + CPW - 1) / CPW;
-    const long long resident = (long long)sm_count() * blocks_per_sm.load() * kRowWarps;
+    const long long resident = (long long)sm_count() * blocks_per_sm * kRowWarps;
     long long n = resident / groups;
     const long long cap = (a.T + 31) / 32;
     if (n > cap) n = cap;

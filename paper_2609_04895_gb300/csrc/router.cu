@@ -1,7 +1,6 @@
 // Host launcher of the router-heads kernel: tensor maps, tile plan, dispatch.
 #include <cudaTypedefs.h>
 
-#include <atomic>
 #include <mutex>
 
 #include "crc_internal.h"
@@ -100,18 +99,15 @@ int launch_router_pair(const crc_problem& p, const uint16_t* w_cat, const CUtens
     c.stream = stream;
     c.attrs = at;
     c.numAttrs = 1;
-    // clusters that fit the GPU at once, -1 before the first call
-    static std::atomic<int> resident{-1};
-    int fit = resident.load();
-    if (fit < 0) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 Cfg::SMEM_BYTES) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&fit, (const void*)kern, &c) != cudaSuccess) {
-            (void)cudaGetLastError();
-            fit = 0;
-        }
-        resident.store(fit);
-    }
+    static PerDevice resident;                 // clusters that fit the GPU at once
+    const int fit = resident.get(current_device(), [&] {
+        int n = 0;
+        if (cuda_status(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             Cfg::SMEM_BYTES)) ||
+            cuda_status(cudaOccupancyMaxActiveClusters(&n, (const void*)kern, &c)))
+            return 0;
+        return n > 0 ? n : -1;
+    });
     if (fit < 1) return CRC_EUNSUPPORTED;
     c.gridDim = dim3((unsigned)(2 * (pa.num_pairs < fit ? pa.num_pairs : fit)));
     CUtensorMap mw;
@@ -156,14 +152,13 @@ int launch_router_t(const crc_problem& p, const uint16_t* hidden, int T_total, i
     a.n_tb = (T_ext + TB - 1) / TB;
     a.num_tiles = p.L * a.n_sb * a.n_tb;
     a.kblocks = (p.d + Cfg::BK - 1) / Cfg::BK;
-    static bool attr_set = false;   // per instantiation
-    if (!attr_set) {
-        const int rc = cuda_status(cudaFuncSetAttribute(
-            router_heads_kernel<NH, H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-            Cfg::SMEM_BYTES));
-        if (rc) return rc;
-        attr_set = true;
-    }
+    static PerDevice ready;
+    const int up = ready.get(current_device(), [&] {
+        return cuda_status(cudaFuncSetAttribute(router_heads_kernel<NH, H>,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                Cfg::SMEM_BYTES)) == CRC_OK;
+    });
+    if (!up) return CRC_ECUDA;
     if constexpr (NH == 128) {
         const int rc = launch_router_pair<H>(p, w_cat, mh, ms, a, stream);
         if (rc != CRC_EUNSUPPORTED) return rc;

@@ -2,7 +2,6 @@
 #pragma once
 
 #include <algorithm>
-#include <atomic>
 
 #include "crc_internal.h"
 #include "short_call.cuh"
@@ -63,20 +62,16 @@ int launch_short_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
     a.tr_mid = trace ? trace->cache_mid_dev : nullptr;
     a.tr_after = trace ? trace->cache_after_dev : nullptr;
     a.tr_sel = trace ? trace->topk_set_dev : nullptr;
+    auto kern = short_call_kernel<NH, V, ALL_VALID, TRACED>;
+    static PerDevice ready;
+    const int up = ready.get(current_device(), [&] {
+        return cuda_status(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                kShortSmem2)) == CRC_OK;
+    });
+    if (!up) return CRC_ECUDA;
     CUtensorMap mh, mw;
     if (!make_hidden_map(&mh, hidden, p.B, T, p.L, p.d, T, a.SB)) return CRC_ECUDA;
     if (!make_weight_map(&mw, w_cat, p.L, 3 * NH, p.d, NH)) return CRC_ECUDA;
-    auto kern = short_call_kernel<NH, V, ALL_VALID, TRACED>;
-    static std::atomic<uint64_t> ready{0};           // devices (of the first 64) set up
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
-    if (bit == 0 || !(ready.load() & bit)) {
-        const int rc = cuda_status(cudaFuncSetAttribute(
-            kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kShortSmem2));
-        if (rc) return rc;
-        ready.fetch_or(bit);
-    }
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)H;

@@ -211,3 +211,62 @@ def test_product_never_imports_the_oracle():
                 txt = open(os.path.join(dirpath, f)).read()
                 assert "import oracle" not in txt and "from oracle" not in txt, f
                 assert "crc_oracle" not in txt, f
+
+
+PER_DEVICE_TEST = r"""
+#include <cassert>
+#include <thread>
+#include <vector>
+
+#include "per_device.h"
+
+int main() {
+    crc::PerDevice p;
+    int calls = 0;
+    auto make = [&](int v) { return [&calls, v] { ++calls; return v; }; };
+    // every device is set up once, with a value of its own
+    assert(p.get(0, make(7)) == 7 && p.get(1, make(9)) == 9 && calls == 2);
+    assert(p.get(0, make(5)) == 7 && p.get(1, make(5)) == 9 && calls == 2);
+    // a failure is not kept, a refusal is, and it stays on its device
+    assert(p.get(2, make(0)) == 0 && p.get(2, make(3)) == 3 && calls == 4);
+    assert(p.get(3, make(-1)) == -1 && p.get(3, make(4)) == -1 && calls == 5);
+    p.set(0, -1);
+    assert(p.get(0, make(7)) == -1 && p.get(1, make(5)) == 9 && calls == 5);
+    // devices past the table, and none at all, ask each time
+    for (int d : {64, 1000, -1}) assert(p.get(d, make(8)) == 8 && p.get(d, make(6)) == 6);
+    p.set(1000, 5);
+    // threads that meet all leave with the value
+    static crc::PerDevice q;
+    std::vector<std::thread> ts;
+    for (int i = 0; i < 8; ++i)
+        ts.emplace_back([] { for (int d = 0; d < 64; ++d) assert(q.get(d, [d] { return d + 1; }) == d + 1); });
+    for (auto& t : ts) t.join();
+    return 0;
+}
+"""
+
+
+def test_setup_is_kept_per_device(tmp_path):
+    """A kernel's attributes and a grid that fits belong to the device they were
+    asked for on (csrc/per_device.h): a second device gets its own."""
+    import subprocess
+    src, exe = tmp_path / "t.cc", tmp_path / "t"
+    src.write_text(PER_DEVICE_TEST)
+    csrc = os.path.join(ROOT, "paper_2609_04895_gb300", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-pthread", "-I", csrc, str(src), "-o", str(exe)],
+                   check=True)
+    subprocess.run([str(exe)], check=True)
+
+
+def test_no_launcher_keeps_its_setup_for_all_devices():
+    """The launchers hold no plain static that a first device's setup would fill in."""
+    csrc = os.path.join(ROOT, "paper_2609_04895_gb300", "csrc")
+    for f in sorted(os.listdir(csrc)):
+        if not f.endswith((".cu", ".cuh")):
+            continue
+        with open(os.path.join(csrc, f)) as fh:
+            for line in fh:
+                m = re.match(r"\s+static (?!const|constexpr|inline)(.*)", line)
+                # process-wide by nature: the driver's entry point, its once flag
+                if m and not re.match(r"(PerDevice|std::once_flag|PFN_\w+) ", m.group(1)):
+                    assert "(" in m.group(1), (f, line)
