@@ -229,6 +229,8 @@ KERNEL_SOURCES = {
     "fused": ["fused.cu", "fused.cuh", "fused_launch.cuh", "fused_n16.cu", "fused_n32.cu",
               "fused_n64.cu", "fused_n128.cu", "router_gemm.cuh", "cache_scan.cuh",
               "crc_device.cuh"],
+    "short": ["short.cu", "short_n128.cu", "short_launch.cuh", "short_call.cuh",
+              "router_gemm.cuh", "cache_scan.cuh", "crc_device.cuh"],
     "router": ["router.cu", "router_gemm.cuh", "router_pair.cuh", "crc_device.cuh"],
     "scan": ["scan.cu", "scan_traced.cu", "scan_launch.cuh", "cache_scan.cuh", "crc_device.cuh"],
     "policy": ["policy.cu", "policy_launch.cuh", "policy_lru.cu", "policy_lfu.cu",
@@ -239,7 +241,7 @@ KERNEL_SOURCES = {
 
 
 def kernel_family(kernel: str) -> str:
-    for fam in ("policy", "fused", "router", "loss"):
+    for fam in ("policy", "fused", "short", "router", "loss"):
         if fam in kernel:
             return fam
     return "scan"
@@ -816,7 +818,10 @@ def rooflines(kt, w, heads, steps, ms, ms_per_step, scan_heads=None, clocks=None
     else:
         flops, bytes_ = algorithmic(w, w.units, heads)
         flops, bytes_ = flops * steps, bytes_ * steps
-        kname = f"fused_route_cache_kernel<{w.N},{heads}>"
+        # a step's calls have one length (but for a streamed run's last chunk), so all of
+        # them or none take the short-call kernel
+        short = kt.get("short", {"launches": 0})["launches"] == kt[dom]["launches"]
+        kname = f"{'short_call' if short else 'fused_route_cache'}_kernel<{w.N},{heads}>"
     t_flop = flops / (tpk * 1e12)
     t_byte = bytes_ / (pk["hbm_gbs"] * 1e9)
     if t_flop >= t_byte:

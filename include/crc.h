@@ -446,11 +446,14 @@ uint64_t crc_launch_count(void);
  * crc_profile_end(), every kernel the library launches is bracketed by two
  * CUDA events recorded on its launching stream.  crc_profile_end()
  * synchronises those events and returns, per kernel kind, the number of
- * launches and their summed device time in milliseconds.  Host-side
- * bookkeeping only; off by default.  Not thread-safe against concurrent
- * library calls from other host threads. */
+ * launches and their summed device time in milliseconds.  FUSED counts every
+ * crc_route_and_cache call that ran as one kernel, and SHORT those among them
+ * that ran as the short-call kernel (counted in both).  Host-side bookkeeping
+ * only; off by default.  Not thread-safe against concurrent library calls from
+ * other host threads. */
 enum { CRC_KERNEL_ROUTER = 0, CRC_KERNEL_SCAN = 1, CRC_KERNEL_STATE = 2, CRC_KERNEL_SYNTH = 3,
        CRC_KERNEL_FUSED = 4, CRC_KERNEL_LOSS = 5, CRC_KERNEL_LOSS_MEANS = 6,
+       CRC_KERNEL_SHORT = 7,
        CRC_KERNEL_KINDS = 8 };
 typedef struct crc_kernel_times {
     uint64_t launches[CRC_KERNEL_KINDS];

@@ -58,7 +58,7 @@ class crc_report(ctypes.Structure):
 
 
 KERNEL_KINDS = {"router": 0, "scan": 1, "state": 2, "synth": 3, "fused": 4, "loss": 5,
-                "loss_means": 6}
+                "loss_means": 6, "short": 7}
 
 
 class crc_kernel_times(ctypes.Structure):

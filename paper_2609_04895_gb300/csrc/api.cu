@@ -519,6 +519,10 @@ int crc_profile_end(crc_kernel_times* out) {
         if (out) {
             out->launches[r.kind] += 1;
             out->ms[r.kind] += ms;
+            if (r.kind == CRC_KERNEL_SHORT) {
+                out->launches[CRC_KERNEL_FUSED] += 1;
+                out->ms[CRC_KERNEL_FUSED] += ms;
+            }
         }
     }
     return rc;

@@ -87,7 +87,7 @@ int launch_short_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
     void* args[] = {(void*)&mh, (void*)&mw, (void*)&a};
     cudaError_t e;
     {
-        ProfScope prof(CRC_KERNEL_FUSED, stream);
+        ProfScope prof(CRC_KERNEL_SHORT, stream);
         e = cudaLaunchKernelExC(&c, (const void*)kern, args);
     }
     note_launch();

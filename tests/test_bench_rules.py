@@ -87,6 +87,33 @@ def test_roofline_arithmetic(monkeypatch):
     assert kernels["fused"]["launches"] == steps
 
 
+def test_one_token_steps_are_named_by_their_own_kernel(monkeypatch):
+    """One-token calls run the short-call kernel: the roofline names it, and a
+    committed traffic figure for it stands on its own sources."""
+    monkeypatch.setattr(bench, "peaks", lambda: (dict(PK), "measured"))
+    w = S.QWEN3_30B.with_(T=1)
+    one = {"ms": 0.03, "launches": 1}
+    kt = {"fused": one, "short": one, "router": {"ms": 0.0, "launches": 0},
+          "scan": {"ms": 0.0, "launches": 0}}
+    roof, _, _ = bench.rooflines(kt, w, 3, 1, 0.03, 0.03)
+    assert roof["kernel"] == "short_call_kernel<128,3>"
+    assert bench.kernel_family(roof["kernel"]) == "short"
+    assert bench.source_hash(roof["kernel"]) != bench.source_hash("fused_route_cache_kernel<128,3>")
+
+
+def test_every_kernel_source_belongs_to_a_family():
+    """The files that define the profiled kernels are among their families' sources."""
+    csrc = os.path.join(ROOT, "paper_2609_04895_gb300", "csrc")
+    listed = set().union(*bench.KERNEL_SOURCES.values())
+    assert all(os.path.exists(os.path.join(csrc, f)) for f in listed)
+    unprofiled = {"scan.cu", "synth.cu", "probe.cu"}       # state init, inputs, failure probe
+    for f in os.listdir(csrc):
+        if f.endswith((".cu", ".cuh")) and f not in unprofiled:
+            with open(os.path.join(csrc, f)) as fh:
+                if "__global__" in fh.read():
+                    assert f in listed, f
+
+
 def test_hbm_bound_roofline_for_n32(monkeypatch):
     monkeypatch.setattr(bench, "peaks", lambda: (dict(PK), "measured"))
     w = S.GPT_OSS_20B

@@ -361,10 +361,12 @@ def test_full_size_workload(C, oracle_lib, w):
 
 # --------------------------------------------------------------------------- #
 FUSED_CASES = [
-    ("tiny", S.TINY),                                               # SB=4, TB=32
-    ("qwen3", S.QWEN3_30B.with_(T=41, L=5)),                        # SB=32, TB=4, ragged T
-    ("gptoss", S.GPT_OSS_20B.with_(B=128, T=23, L=3, d=576)),       # 4 stream groups
-    ("r0", S.QWEN3_30B.with_(B=40, T=19, L=4, R=0, C=16)),          # 2 heads, partial group
+    # every case is two calls, of a third and two thirds of its tokens: those of up to 64
+    # run on the short-call kernel, the others on the persistent one
+    ("tiny", S.TINY),                                               # 85 | 171: 128-token tiles
+    ("qwen3", S.QWEN3_30B.with_(T=41, L=5)),                        # 13 | 28, 9 and 4 streams a tile
+    ("gptoss", S.GPT_OSS_20B.with_(B=128, T=23, L=3, d=576)),       # 7 | 16, a ragged last group
+    ("r0", S.QWEN3_30B.with_(B=40, T=19, L=4, R=0, C=16)),          # 6 | 13, 2 heads, ragged groups
     ("n64-one-layer", S.TINY.with_(N=64, K=3, C=9, R=5, B=6, T=50, L=1, d=192)),
     ("k1", S.TINY.with_(K=1, C=2, R=2, B=9, T=33)),
     # 128-token tiles of one stream: N = 128 runs on CTA pairs when B is even
@@ -377,7 +379,7 @@ FUSED_CASES = [
 
 @pytest.mark.parametrize("name,w", FUSED_CASES, ids=[c[0] for c in FUSED_CASES])
 def test_fused_kernel_equals_pair(C, name, w):
-    """route_and_cache with a workspace large enough for the fused kernel
+    """route_and_cache as one kernel (a workspace large enough for the fused one)
     equals route_scores + cache_scan bit for bit, over two calls that continue
     the same streams: without a trace, and with the fused kernel writing its
     per-access trace (Top-K set, misses, proactive loads, the cache after the
@@ -400,11 +402,13 @@ def test_fused_kernel_equals_pair(C, name, w):
         C.route_and_cache(p, hc, W, st_fused, None, workspace=ws)
         kt = C.crc_profile_end()
         assert kt["fused"]["launches"] == 1 and kt["router"]["launches"] == 0
+        assert kt["short"]["launches"] == int(n <= 64)
         tf = C.Trace.alloc(p, n, caches=True, rank_order=False, topk_set=True)
         C.crc_profile_begin()
         C.route_and_cache(p, hc, W, st_traced, tf, workspace=ws)
         kt = C.crc_profile_end()
         assert kt["fused"]["launches"] == 1 and kt["router"]["launches"] == 0
+        assert kt["short"]["launches"] == int(n <= 64)
         tr_pair.append(tp)
         tr_fused.append(tf)
         t0 += n
