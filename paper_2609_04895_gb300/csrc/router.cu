@@ -73,9 +73,16 @@ bool make_scores_map(CUtensorMap* m, float* scores, int B, int T_ext, int L, int
 namespace {
 
 // The launch on CTA pairs.  A layer's tiles are paired in order; an odd last
-// one has an idle partner, which costs up to half a tile's time a layer, so
-// pairs are taken when that is little or when the whole call is one wave
-// anyway.  CRC_EUNSUPPORTED: the single-CTA kernel takes the call.
+// one has an idle partner.  What decides is the rounds of tiles that an SM runs:
+// a pair's round takes 0.86 to 0.96 of a single CTA's for d >= 2048 (0.87 to 0.92
+// at d = 7168), so pairs pay unless idle partners add more than one round in
+// sixteen.  Us, single / pairs, three heads: 48 layers of 9 tiles, 3 rounds
+// against 4, 82 / 95; of 15, 5 against 6, 129 / 139; 94 layers of 27, 17 against
+// 18, 425 / 419.  Shorter rows are bound by the epilogue and gain nothing
+// (d = 1024, equal rounds: 0.95 to 1.06), and a call of one round has the
+// cluster's set-up to make up for as well (d = 2048 0.94 to 1.08, d = 1024 1.00
+// to 1.09, d = 4096 0.87 to 1.02).  CRC_EUNSUPPORTED: the single-CTA kernel
+// takes the call.
 template <int H>
 int launch_router_pair(const crc_problem& p, const uint16_t* w_cat, const CUtensorMap& mh,
                        const CUtensorMap& ms, const RouterArgs& a, cudaStream_t stream) {
@@ -85,7 +92,11 @@ int launch_router_pair(const crc_problem& p, const uint16_t* w_cat, const CUtens
     const int tiles = a.n_sb * a.n_tb;
     pa.pairs_per_layer = (tiles + 1) / 2;
     pa.num_pairs = p.L * pa.pairs_per_layer;
-    if (tiles % 2 != 0 && tiles < 9 && 2 * pa.num_pairs > sm_count()) return CRC_EUNSUPPORTED;
+    const int sms = sm_count(), pairs = sms / 2;
+    const int rounds = (a.num_tiles + sms - 1) / sms;
+    const int pair_rounds = pairs > 0 ? (pa.num_pairs + pairs - 1) / pairs : 0;
+    if (p.d < (rounds > 1 ? 2048 : 4096) || pairs < 1 || 15ll * pair_rounds > 16ll * rounds)
+        return CRC_EUNSUPPORTED;
     auto kern = router_pair_kernel<H>;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;

@@ -1,7 +1,8 @@
-"""Router heads of N = 128 on CTA pairs: a layer's tiles pair up whatever their
-number, so the scores of a call equal, bit for bit, those of calls on parts of
-it whose tiles pair up differently or not at all (few odd tiles a layer run on
-one CTA each), and match an fp64 softmax.
+"""Router heads of N = 128, on CTA pairs and on one CTA a tile (rows shorter than
+2048, or than 4096 in a call of one round, or where pairs would take more
+rounds): a layer's tiles pair up whatever their number, so the scores of a call
+equal, bit for bit, those of calls on parts of it whose tiles pair up
+differently or not at all, and match an fp64 softmax.
 """
 import pytest
 
@@ -23,16 +24,17 @@ def C():
 
 
 # (layers, streams, tokens): one tile a layer, two, three (partner idle, one
-# wave), three of more than a wave (single CTAs), nine and more, tiles of
-# several streams, ragged lengths
+# round either way), three of more rounds on pairs (single CTAs), nine and more,
+# tiles of several streams, ragged lengths
 SIZES = [(3, 1, 100), (3, 2, 128), (3, 3, 128), (60, 3, 70), (20, 9, 130), (17, 5, 257),
          (4, 40, 7), (3, 300, 1), (2, 1, 1)]
 
 
 @pytest.mark.parametrize("L,B,T", SIZES, ids=lambda v: str(v))
 @pytest.mark.parametrize("heads", [3, 2])
-def test_pairs_equal_parts(C, L, B, T, heads):
-    w = S.QWEN3_30B.with_(L=L, B=B, T=T, d=328)
+@pytest.mark.parametrize("d", [328, 2056, 4104])
+def test_pairs_equal_parts(C, L, B, T, heads, d):
+    w = S.QWEN3_30B.with_(L=L, B=B, T=T, d=d)
     W = C.synth_weights(L, w.N, w.d, seed=3)
     h, _ = C.synth_hidden(B, T, L, w.d, seed=4)
     mark = -7.0
@@ -53,6 +55,6 @@ def test_pairs_equal_parts(C, L, B, T, heads):
         z = h[:, :, l].double() @ W[l].double().t()
         ref = torch.softmax(z.view(B, T, 3, w.N), dim=-1)[:, :, :heads]
         err = (full[:, :, l, :heads].double() - ref).abs() / ref
-        # fp32 sums of 328 products and the SFU exponential, as for the other
-        # router tests
+        # fp32 sums of d products and the SFU exponential, as for the other router
+        # tests (d up to 2880)
         assert float(err.max()) <= 2.5e-4
