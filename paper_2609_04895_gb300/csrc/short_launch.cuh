@@ -9,9 +9,7 @@
 namespace crc {
 
 // Shared memory a CTA may take so that two (twelve warps each) or three (eight
-// warps each) fit an SM: 80 registers a thread allow both.  Three when the
-// call has more CTAs than two an SM: they wait on their chains' steps, and
-// more of them overlap.
+// warps each) fit an SM: 80 registers a thread allow both.
 constexpr int kShortSmem2 = 113 * 1024;
 constexpr int kShortSmem3 = 75 * 1024;
 
@@ -19,6 +17,33 @@ constexpr int kShortSmem3 = 75 * 1024;
 inline bool trace_wanted(const crc_trace* t) {
     return t && (t->misses_dev || t->proactive_dev || t->cache_mid_dev || t->cache_after_dev ||
                  t->topk_set_dev);
+}
+
+// Where a call is faster on the short-call kernel than on the persistent fused
+// one, by the waves of clusters it would run in with two CTAs an SM and with
+// three (times in us, persistent / short, traced calls on one GB300):
+//  - one or two tokens: the persistent kernel's tiles are then one layer's whole
+//    work and its scan items one step long.  N = 128, d = 2048, 48 layers: T = 1,
+//    B = 64 56 / 31, B = 1024 348 / 152; N = 32: B = 1024 150 / 73; d = 4096:
+//    T = 2, B = 256 243 / 222.  Not two tokens of wide rows in several waves,
+//    when the hidden rows that the heads' CTAs read again cost more (N = 128,
+//    d = 7168, T = 2, untraced: B = 128 140 / 118 in one wave, B = 200 171 / 201,
+//    B = 600 384 / 493).
+//  - up to four unless d is large, for the same reason (T = 4, B = 128:
+//    d = 2048 109 / 95, d = 4096 197 / 229), nor four tokens of 128 experts in
+//    more than three waves (T = 4, B = 300, untraced: 152 / 162).
+//  - up to 64 tokens when every cluster is resident at once, two CTAs an SM
+//    (three for N = 128): with a second wave the chains' steps, which take most
+//    of such a call, come twice (N = 128: T = 24, B = 13 91 / 63; T = 16, B = 16
+//    60 / 47; T = 16, B = 64 128 / 154).  Untraced calls of up to 32 experts only
+//    to 32 tokens (T = 64, B = 1: 57 / 57), longer ones not at all: the
+//    persistent kernel runs several tiles' chains side by side.
+inline bool short_call_takes(const crc_problem& p, int T, bool traced, int waves2, int waves3) {
+    const bool one_wave = waves2 <= 1 || (p.N == 128 && waves3 <= 1);
+    if (T <= 1) return true;
+    if (T <= 2) return one_wave || p.N < 128 || p.d <= 4096;
+    if (T <= 4 && p.d <= 3072) return T <= 3 || p.N < 128 || waves2 <= 3;
+    return T <= (traced || p.N > 32 ? 64 : 32) && one_wave;
 }
 
 template <int NH, int V, bool ALL_VALID, bool TRACED>
@@ -51,7 +76,20 @@ int launch_short_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
     a.tr_at = a.sel_at + own_rows * 32;
     const int after = a.tr_at + (TRACED ? own_rows * 34 : 0);
     const int fixed = 1024 + Cfg::TAIL_BYTES;
-    const bool three = grid > 2 * sm_count() && fixed + after <= kShortSmem3;
+    // Waves of clusters.  Clusters of three leave a twentieth of the SMs' places
+    // empty: with three CTAs an SM 144 of them run in one wave, 150 in two.
+    const int places = std::max(1, sm_count() * 19 / 20);
+    const int waves2 = (grid + 2 * places - 1) / (2 * places);
+    const int waves3 =
+        fixed + after <= kShortSmem3 ? (grid + 3 * places - 1) / (3 * places) : waves2;
+    if (!short_call_takes(p, T, TRACED, waves2, waves3)) return CRC_EUNSUPPORTED;
+    // Three CTAs an SM when that saves enough waves: they share the SM's loads,
+    // so a wave takes 1.3 to 1.45 times one of two (1.6 for N = 64, whose three
+    // have fewer bytes in flight).  One token, us, two / three an SM: N = 128,
+    // d = 2048, B = 300, waves 2 / 1 65 / 50; B = 400, 2 / 2 70 / 84; B = 600,
+    // 3 / 2 100 / 93; N = 64, d = 5120, B = 400, 2 / 1 73 / 67; B = 600, 2 / 2
+    // 83 / 122; B = 1024, 3 / 2 128 / 139.
+    const bool three = NH == 64 ? 8 * waves3 <= 5 * waves2 : 4 * waves3 <= 3 * waves2;
     const int room = (three ? kShortSmem3 : kShortSmem2) - fixed - overrun;
     a.stages = std::max(1, std::min({kShortMaxStages, a.kblocks, room / a.stage_bytes}));
     a.tail = (std::max(a.stages * a.stage_bytes + overrun, after) + 1023) & ~1023;

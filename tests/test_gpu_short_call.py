@@ -37,11 +37,9 @@ SIZES = [(1, 1), (127, 1), (128, 1), (129, 1), (300, 1), (43, 3), (7, 5), (3, 42
          (5, 64), (1, 65)]
 
 
-@pytest.mark.parametrize("shape", SHAPES, ids=str)
-@pytest.mark.parametrize("B,T", SIZES, ids=lambda v: str(v))
-@pytest.mark.parametrize("traced", [True, False], ids=["traced", "untraced"])
-def test_short_calls_equal_pair(C, shape, B, T, traced):
-    w = SHAPES[shape].with_(B=B)
+def run_short_calls(C, w, traced, short_kernel):
+    """Three successive calls of w.T tokens on one state against the pair's."""
+    B, T = w.B, w.T
     p = C.problem_of(w)
     W = C.synth_weights(w.L, w.N, w.d, seed=3)
     ws = torch.empty(C.crc_fused_workspace_bytes(p), dtype=torch.uint8, device="cuda")
@@ -52,7 +50,10 @@ def test_short_calls_equal_pair(C, shape, B, T, traced):
         h, carry = C.synth_hidden(B, T, w.L, w.d, seed=4, t0=call * T, carry=carry)
         trs = C.Trace.alloc(p, T, caches=True, rank_order=False, topk_set=True)
         trp = C.Trace.alloc(p, T, caches=True, rank_order=False, topk_set=True)
+        C.crc_profile_begin()
         C.route_and_cache(p, h, W, short, trs if traced else None, workspace=ws)
+        kt = C.crc_profile_end()
+        assert kt["fused"]["launches"] == 1 and kt["short"]["launches"] == int(short_kernel)
         scores = torch.zeros((B, T, w.L, 3, w.N), device="cuda")
         C.cache_scan(p, C.route_scores(p, h, W, heads=heads, out=scores), pair, trp)
         if traced:
@@ -64,6 +65,84 @@ def test_short_calls_equal_pair(C, shape, B, T, traced):
     for name in ("cache_bits", "chain_counters"):
         assert (a[name] == b[name]).all(), name
     assert (a["retention"].view("u4") == b["retention"].view("u4")).all()
+
+
+# Calls of more clusters than two CTAs an SM hold, where three an SM (of eight
+# warps) save a wave, and one on the other side of that line
+THREE = {
+    "n128-24": S.QWEN3_30B.with_(L=48, B=13, T=24, d=256),
+    "n128-24-two": S.QWEN3_30B.with_(L=30, B=13, T=24, d=256),
+    "n128-one": S.QWEN3_30B.with_(L=48, B=300, T=1, d=520),
+    "n128-r0": S.QWEN3_30B.with_(L=90, B=150, T=1, d=200, R=0, C=16),
+    "n64": S.TINY.with_(N=64, K=6, C=12, R=3, L=30, B=400, T=1, d=264),
+    "n32": S.GPT_OSS_20B.with_(L=24, B=600, T=1, d=200),
+    "n16": S.TINY.with_(L=48, B=300, T=2, d=136),
+}
+
+
+@pytest.mark.parametrize("name", THREE, ids=str)
+@pytest.mark.parametrize("traced", [True, False], ids=["traced", "untraced"])
+def test_short_calls_of_many_clusters(C, name, traced):
+    run_short_calls(C, THREE[name], traced, True)
+
+
+def test_one_state_over_short_and_persistent_calls(C):
+    """A serving loop's mix on one state: single tokens, chunks and long calls in
+    turn, traced and not, against one scan of the same scores in the same pieces."""
+    w = S.QWEN3_30B.with_(B=6, L=3, d=256)
+    p = C.problem_of(w)
+    W = C.synth_weights(w.L, w.N, w.d, seed=3)
+    ws = torch.empty(C.crc_fused_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    mixed, pair = C.State(p), C.State(p)
+    carry, t0 = None, 0
+    for i, T in enumerate([1, 150, 1, 24, 2, 200, 64, 1, 66, 3]):
+        h, carry = C.synth_hidden(w.B, T, w.L, w.d, seed=4, t0=t0, carry=carry)
+        trm = C.Trace.alloc(p, T, caches=True, rank_order=False, topk_set=True)
+        trp = C.Trace.alloc(p, T, caches=True, rank_order=False, topk_set=True)
+        C.crc_profile_begin()
+        C.route_and_cache(p, h, W, mixed, trm if i % 3 else None, workspace=ws)
+        assert C.crc_profile_end()["short"]["launches"] == int(T <= 64)
+        C.cache_scan(p, C.route_scores(p, h, W), pair, trp)
+        if i % 3:
+            for name in ("misses", "proactive", "cache_mid", "cache_after", "topk_set"):
+                assert torch.equal(getattr(trm, name), getattr(trp, name)), (i, name)
+        t0 += T
+    a = mixed.read(want_caches=True, want_retention=True, want_chain_counters=True)
+    b = pair.read(want_caches=True, want_retention=True, want_chain_counters=True)
+    assert a["error"] == 0 and a["tokens"] == t0
+    for name in ("cache_bits", "chain_counters"):
+        assert (a[name] == b[name]).all(), name
+    assert (a["retention"].view("u4") == b["retention"].view("u4")).all()
+
+
+def test_aborted_short_call_does_not_advance_the_state(C):
+    """A call that finds its abort word set (as one of its waits sets it when it
+    runs out) leaves the token counter and the carry slot where they were and
+    clears the word, so the next call runs."""
+    w = SHAPES["n128"].with_(B=4)
+    p = C.problem_of(w)
+    st = C.State(p)
+    W = C.synth_weights(w.L, w.N, w.d, seed=3)
+    ws = torch.empty(C.crc_fused_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    h, _ = C.synth_hidden(4, 1, w.L, w.d, seed=4)
+    C.route_and_cache(p, h, W, st, None, workspace=ws)
+    head = st.buf[:256].view(torch.int32)
+    before = head.cpu()
+    word = 15                                         # the header's abort word
+    head[word] = 1
+    C.route_and_cache(p, h, W, st, None, workspace=ws)
+    assert torch.equal(head.cpu(), before)            # the word cleared, nothing else moved
+    C.route_and_cache(p, h, W, st, None, workspace=ws)
+    assert st.read()["tokens"] == 2
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=str)
+@pytest.mark.parametrize("B,T", SIZES, ids=lambda v: str(v))
+@pytest.mark.parametrize("traced", [True, False], ids=["traced", "untraced"])
+def test_short_calls_equal_pair(C, shape, B, T, traced):
+    w = SHAPES[shape].with_(B=B, T=T)
+    # untraced calls of few experts leave the short-call kernel at 32 tokens, others at 64
+    run_short_calls(C, w, traced, T <= (64 if traced or w.N > 32 else 32))
 
 
 def test_short_call_on_another_problems_state(C):
