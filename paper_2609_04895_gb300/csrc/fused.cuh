@@ -451,14 +451,18 @@ struct FusedCfg {
     // issue slots from the epilogue.  Three heads of 128 experts: 6 (64 x 1024
     // tokens, 5 to 8 warps within 2 %, 4 10 % slower; R = 8 the same).  Fewer
     // columns or no Spatio head mean shorter tiles: 8 (N = 32, 64 x 1000: 6
-    // 1483 us, 8 1361; R = 0, 48 x 777: 1714 and 1608).  The kernel's roles do
-    // not depend on the count: every warp past the GEMM warps scans.
+    // 1483 us, 8 1361; R = 0, 48 x 777: 1714 and 1608).  So do blocks of few
+    // tokens, whose items' start and end weigh more than their steps: 8 (N = 128,
+    // R = 8, d = 4096, 300 streams x 3 tokens: 6 360 us, 8 307; traced 431 and
+    // 363; d = 2048, R = 4, 128 x 8: 135 and 118).  The kernel's roles do not
+    // depend on the count: every warp past the GEMM warps scans.
     static constexpr int SCAN_WARPS = 6;
     static constexpr int SCAN_WARPS_WIDE = 8;
     static constexpr int THREADS = 32 * (GEMM_WARPS + SCAN_WARPS);
     static constexpr int MAX_THREADS = 32 * (GEMM_WARPS + SCAN_WARPS_WIDE);
-    static int threads_for(int R) {
-        return 32 * (GEMM_WARPS + (NH == 128 && R > 0 ? SCAN_WARPS : SCAN_WARPS_WIDE));
+    static int threads_for(int R, int TB) {
+        const bool few = NH == 128 && R > 0 && TB > 16;
+        return 32 * (GEMM_WARPS + (few ? SCAN_WARPS : SCAN_WARPS_WIDE));
     }
     static constexpr int B_ROWS = PAIR ? RC::NCOL / 2 : RC::NCOL;        // weight rows per CTA
     static constexpr int B_BOX_ROWS = PAIR ? RC::NCH / 2 : RC::B_BOX_ROWS;

@@ -165,7 +165,7 @@ int launch_fused_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
     a.tr_after = trace ? trace->cache_after_dev : nullptr;
     a.tr_sel = trace ? trace->topk_set_dev : nullptr;
     void* args[] = {(void*)&mh, (void*)&mw, (void*)&a};
-    const int threads = Cfg::threads_for(p.R);
+    const int threads = Cfg::threads_for(p.R, f.TB);
     cudaError_t e;
     if (PAIR) {
         cudaLaunchAttribute at[2];
