@@ -44,9 +44,21 @@ inline double tile_cost(int N, int R, int tb) {
     return cost[N <= 32 ? 0 : N <= 64 ? 1 : R > 0 ? 2 : 3][i];
 }
 
+// DRAM time of a layer, in tiles, when the weights do not stay in L2 from one
+// token block to the next: the hidden states once and the weights once a block,
+// against a tile's time at 0.78 of the bf16 peak or, for few columns, that of
+// its hidden rows.
+inline double layer_bytes_cost(int columns, int n_bg, int n_tb) {
+    const double flop_bound = columns / 216.0;           // a tile's MMAs : its hidden rows
+    return n_tb * (n_bg + columns / 128.0) / (flop_bound > 1.0 ? flop_bound : 1.0);
+}
+constexpr double kL2Bytes = 129e6;
+
 // Tokens of a block: all of a shorter call; otherwise the cheapest by tiles a
 // layer times a tile's cost, an N = 128 plan whose tiles do not pair up (see
-// launch_fused_pair) counting 12 % more.  With fewer chains than about the scan
+// launch_fused_pair) counting 12 % more, and no less than the DRAM time of
+// weights that L2 does not hold (94 layers, d = 4096, 296 MB of them, 13 streams
+// x 200 tokens: blocks of 16 986 us, 32 811, 64 846, 128 859).  With fewer chains than about the scan
 // warps (1,024), or rows short enough that a tile's GEMM takes less than its
 // scan (d < 1024), the chains' steps bound the call, not its tiles, and longer
 // items are better (N = 16, d = 256, 256 x 500: 327 us, with TB = 16 358).
@@ -61,6 +73,9 @@ inline int block_tokens(const crc_problem& p, int T) {
         const int n_bg = (p.B + 128 / c - 1) / (128 / c);
         double cost = (double)n_bg * ((T + c - 1) / c) * tile_cost(p.N, p.R, c);
         if (p.N == 128 && n_bg % 2 != 0) cost *= 1.12;
+        const int columns = (p.R > 0 ? 3 : 2) * p.N;
+        if (2.0 * p.L * columns * p.d > kL2Bytes)
+            cost = std::max(cost, layer_bytes_cost(columns, n_bg, (T + c - 1) / c));
         if (c == 128 || cost < best) {
             best = cost;
             tb = c;
