@@ -351,6 +351,7 @@ __global__ void __launch_bounds__(192, 1)
             const int l = tile / tiles_per_layer;
             const int r = tile % tiles_per_layer;
             const int sb = r / a.n_tb, tb = r % a.n_tb;
+            const bool ok = CRC_IN_BOUNDS(l < a.L && sb < a.n_sb && tb < a.n_tb, a.err);
             const uint32_t tbase =
                 tmem_base + (uint32_t)(acc * Cfg::ACC_COLS) + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
@@ -391,7 +392,7 @@ __global__ void __launch_bounds__(192, 1)
                                                               z[32 * c + 4 * j + 3]);
                         fence_proxy_async_smem();
                         __syncwarp();
-                        if (lane == 0) {
+                        if (lane == 0 && ok) {
                             tma_store_5d(&tmap_s, sbuf, c * 32, h, l, tok0, str0);
                             bulk_commit();
                         }
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(192, 1)
                 } else {
                     const int b = sb * a.SB + row / a.TB;
                     const int t = tb * a.TB + row % a.TB;
-                    if (b < a.B && t < a.T_ext) {
+                    if (ok && b < a.B && t < a.T_ext) {
                         float4* o = reinterpret_cast<float4*>(
                             a.scores + (((size_t)b * a.T_ext + t) * a.L + l) * (size_t)(3 * NH) +
                             h * NH);

@@ -211,8 +211,9 @@ __global__ void __launch_bounds__(RouterPairCfg<H>::THREADS, 1)
             tc_fence_after();
             const int l = q / pa.pairs_per_layer;
             const int r = 2 * (q % pa.pairs_per_layer) + (int)rank;
-            const bool real = r < tiles_per_layer;
             const int sb = r / a.n_tb, tb = r % a.n_tb;
+            const bool real = r < tiles_per_layer &&
+                              CRC_IN_BOUNDS(l < a.L && sb < a.n_sb && tb < a.n_tb, a.err);
             const int row0 = quarter * 32;
             const int str0 = sb * a.SB + row0 / a.TB;
             const int tok0 = tb * a.TB + row0 % a.TB;

@@ -207,7 +207,12 @@ __global__ void __launch_bounds__(ShortCfg<NH>::MAX_THREADS, 2)
     const int lw = rank == 2 ? (l > 0 ? l - 1 : a.L - 1) : l;   // layer of this CTA's head
     StateHeader* hdr = reinterpret_cast<StateHeader*>(a.state);
     uint32_t* err = &hdr->error;
-    const bool in_bounds = CRC_IN_BOUNDS(l < a.L && b0 < a.B && lw < a.L && n_str * a.T <= 128, err);
+    const bool in_bounds = CRC_IN_BOUNDS(
+        l < a.L && b0 < a.B && lw < a.L && n_str * a.T <= 128 && n_str * a.T * ROW * 4 <= a.sel_at &&
+            n_own * a.T * 32 <= a.tr_at - a.sel_at &&
+            (!TRACED || a.tr_at + n_own * a.T * 34 <= a.tail) && a.tr_at <= a.tail &&
+            a.stages * a.stage_bytes <= a.tail,
+        err);
     auto timed_out = [&] {
         latch_error(err, CRC_ETIMEOUT);
         atomicExch(fail, 1u);
@@ -331,6 +336,7 @@ __global__ void __launch_bounds__(ShortCfg<NH>::MAX_THREADS, 2)
     auto load_chain = [&](int j) {
         Loaded q;
         const int chain = (b0 + rank + H * j) * L + l;
+        if (!CRC_IN_BOUNDS(b0 + rank + H * j < a.B, err)) return Loaded{};
         const ChainState& cs = chains[chain];
         q.bits = lane_bits<V>(cs.bits, lane, N);
         q.aT = load_vec<V>(retention + (size_t)chain * N + e0, has);
@@ -542,7 +548,9 @@ __global__ void __launch_bounds__(ShortCfg<NH>::MAX_THREADS, 2)
         __syncthreads();
         for (int i = warp; go && i < n_own * T; i += warps) {
             const int t = i % T;
-            const size_t unit = ((size_t)(b0 + rank + H * (i / T)) * T + t) * L + l;
+            const int b = b0 + rank + H * (i / T);
+            if (!CRC_IN_BOUNDS(b < a.B && l < L, err)) continue;
+            const size_t unit = ((size_t)b * T + t) * L + l;
             const uint32_t sets = sets_s[i * 32 + lane], sel = sel_s[i * 32 + lane];
             if (a.tr_mid) store_cache_words<V>(sets & 15u, lane, N, a.tr_mid + unit * NW);
             if (a.tr_after) store_cache_words<V>(sets >> 4, lane, N, a.tr_after + unit * NW);

@@ -21,6 +21,18 @@ CASES = {
     "pairs-n128": S.QWEN3_30B.with_(B=4, T=300, L=3, d=256),
     "n32": S.GPT_OSS_20B.with_(B=8, T=150, L=3, d=576),
     "r0-one-cta": S.QWEN3_30B.with_(B=3, T=70, L=2, R=0, C=16, d=256),
+    # the short-call kernel: two CTAs an SM, three, one token of two heads
+    "short-n16": S.TINY.with_(B=9, T=40),
+    "short-n128-three": S.QWEN3_30B.with_(B=13, T=24, L=40, d=256),
+    "short-r0-one-token": S.QWEN3_30B.with_(B=130, T=1, L=5, R=0, C=16, d=200),
+    # the persistent kernel's short blocks: 8 tokens on CTA pairs and on single CTAs, and
+    # the longer calls that take blocks of 16 to 64
+    "blocks-of-8-pairs": S.QWEN3_30B.with_(B=128, T=8, L=24, d=64),
+    "blocks-of-8": S.QWEN3_30B.with_(B=100, T=7, L=32, d=64),
+    "blocks-n16": S.TINY.with_(B=128, T=67, L=8, d=1024),
+    "blocks-pairs": S.QWEN3_30B.with_(B=115, T=66, L=9, d=1024),
+    # router heads on CTA pairs (d >= 2048), an odd number of tiles a layer
+    "router-pairs-odd": S.QWEN3_30B.with_(B=17, T=128, L=16, d=2048),
 }
 
 
@@ -33,7 +45,7 @@ def run_cases(C) -> dict:
         h, _ = C.synth_hidden(w.B, w.T, w.L, w.d, seed=52, rho_t=w.rho_t, rho_l=w.rho_l)
         heads = 3 if w.R > 0 else 2
         runs = {}
-        # the fused kernel without and with its trace
+        # one kernel for the call, without and with its trace
         wsf = torch.empty(C.crc_fused_workspace_bytes(p), dtype=torch.uint8, device="cuda")
         st = C.State(p)
         C.route_and_cache(p, h, W, st, None, workspace=wsf)
