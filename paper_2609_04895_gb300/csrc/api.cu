@@ -284,11 +284,12 @@ int crc_route_and_cache(const crc_problem* p, const uint16_t* hidden_dev,
     // the scores of one token have to fit, unless the fused kernel's ring does
     const size_t per_token = crc_workspace_bytes(p, 1);
     const long long fit = (long long)(workspace_bytes / per_token);
-    if (fit < 1 && workspace_bytes < fused_workspace_bytes(*p)) return CRC_EINVAL;
+    const bool persistent = workspace_bytes >= fused_workspace_bytes(*p);
+    if (fit < 1 && !persistent) return CRC_EINVAL;
     // the fused kernels know the Top-K as a set only: a trace in rank order
     // takes the two-kernel path
     if (!(trace && trace->topk_dev)) {
-        rc = launch_short(*p, hidden_dev, w_cat_dev, T, state_dev, trace, s);
+        rc = launch_short(*p, hidden_dev, w_cat_dev, T, state_dev, trace, persistent, s);
         if (rc != CRC_EUNSUPPORTED) return rc;
         rc = launch_fused(*p, hidden_dev, w_cat_dev, T, state_dev, workspace_dev, workspace_bytes,
                           trace, s);

@@ -70,10 +70,16 @@ int launch_fused_n32(const crc_problem& p, const uint16_t* hidden, const uint16_
 int launch_fused_n64(const crc_problem& p, const uint16_t* hidden, const uint16_t* w_cat, int T,
                      void* state, void* workspace, const crc_trace* trace,
                      cudaStream_t stream);
+// Any array of the trace that the one-kernel calls write.
+inline bool trace_wanted(const crc_trace* t) {
+    return t && (t->misses_dev || t->proactive_dev || t->cache_mid_dev || t->cache_after_dev ||
+                 t->topk_set_dev);
+}
 // Short calls (short.cu): one cluster per (layer, stream group), no workspace;
-// CRC_EUNSUPPORTED for calls it does not take.
+// CRC_EUNSUPPORTED for calls it does not take.  persistent: the workspace has
+// room for the persistent fused kernel, which takes those.
 int launch_short(const crc_problem& p, const uint16_t* hidden, const uint16_t* w_cat, int T,
-                 void* state, const crc_trace* trace, cudaStream_t stream);
+                 void* state, const crc_trace* trace, bool persistent, cudaStream_t stream);
 // Cache scan under a comparison policy (policy_scan.cuh).
 int launch_policy_scan(const crc_problem& p, const float* scores, int T, void* state,
                        const crc_trace* trace, int trace_T, int trace_t0, int policy,

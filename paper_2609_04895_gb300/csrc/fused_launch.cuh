@@ -279,13 +279,11 @@ template <int NH, int V, bool ALL_VALID>
 int launch_fused_for_n(const crc_problem& p, const uint16_t* hidden, const uint16_t* w_cat,
                        int T, void* state, void* workspace, const crc_trace* trace,
                        cudaStream_t stream) {
-    const bool traced = trace && (trace->misses_dev || trace->proactive_dev ||
-                                  trace->cache_mid_dev || trace->cache_after_dev ||
-                                  trace->topk_set_dev);
-    return traced ? launch_fused_mode<NH, V, ALL_VALID, true>(p, hidden, w_cat, T, state,
-                                                              workspace, trace, stream)
-                  : launch_fused_mode<NH, V, ALL_VALID, false>(p, hidden, w_cat, T, state,
-                                                               workspace, nullptr, stream);
+    return trace_wanted(trace)
+               ? launch_fused_mode<NH, V, ALL_VALID, true>(p, hidden, w_cat, T, state, workspace,
+                                                           trace, stream)
+               : launch_fused_mode<NH, V, ALL_VALID, false>(p, hidden, w_cat, T, state, workspace,
+                                                            nullptr, stream);
 }
 
 }  // namespace crc

@@ -13,12 +13,6 @@ namespace crc {
 constexpr int kShortSmem2 = 113 * 1024;
 constexpr int kShortSmem3 = 75 * 1024;
 
-// Any array of the trace that the fused kernels write.
-inline bool trace_wanted(const crc_trace* t) {
-    return t && (t->misses_dev || t->proactive_dev || t->cache_mid_dev || t->cache_after_dev ||
-                 t->topk_set_dev);
-}
-
 // Where a call is faster on the short-call kernel than on the persistent fused
 // one, by the waves of clusters it would run in with two CTAs an SM and with
 // three (times in us, persistent / short, traced calls on one GB300):
@@ -38,9 +32,14 @@ inline bool trace_wanted(const crc_trace* t) {
 //    60 / 47; T = 16, B = 64 128 / 154).  Untraced calls of up to 32 experts only
 //    to 32 tokens (T = 64, B = 1: 57 / 57), longer ones not at all: the
 //    persistent kernel runs several tiles' chains side by side.
-inline bool short_call_takes(const crc_problem& p, int T, bool traced, int waves2, int waves3) {
+// Without room for the persistent kernel the choice is the router's and the
+// scan's launches, a chunk of tokens at a time: up to two tokens, and four of
+// rows that are not wide, are then taken in any number of waves.
+inline bool short_call_takes(const crc_problem& p, int T, bool traced, bool persistent,
+                             int waves2, int waves3) {
     const bool one_wave = waves2 <= 1 || (p.N == 128 && waves3 <= 1);
     if (T <= 1) return true;
+    if (!persistent && (T <= 2 || (T <= 4 && p.d <= 3072))) return true;
     if (T <= 2) return one_wave || p.N < 128 || p.d <= 4096;
     if (T <= 4 && p.d <= 3072) return T <= 3 || p.N < 128 || waves2 <= 3;
     return T <= (traced || p.N > 32 ? 64 : 32) && one_wave;
@@ -48,7 +47,7 @@ inline bool short_call_takes(const crc_problem& p, int T, bool traced, int waves
 
 template <int NH, int V, bool ALL_VALID, bool TRACED>
 int launch_short_t(const crc_problem& p, const uint16_t* hidden, const uint16_t* w_cat, int T,
-                   void* state, const crc_trace* trace, cudaStream_t stream) {
+                   void* state, const crc_trace* trace, bool persistent, cudaStream_t stream) {
     using Cfg = ShortCfg<NH>;
     ShortArgs a;
     a.state = static_cast<uint8_t*>(state);
@@ -82,7 +81,7 @@ int launch_short_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
     const int waves2 = (grid + 2 * places - 1) / (2 * places);
     const int waves3 =
         fixed + after <= kShortSmem3 ? (grid + 3 * places - 1) / (3 * places) : waves2;
-    if (!short_call_takes(p, T, TRACED, waves2, waves3)) return CRC_EUNSUPPORTED;
+    if (!short_call_takes(p, T, TRACED, persistent, waves2, waves3)) return CRC_EUNSUPPORTED;
     // Three CTAs an SM when that saves enough waves: they share the SM's loads,
     // so a wave takes 1.3 to 1.45 times one of two (1.6 for N = 64, whose three
     // have fewer bytes in flight).  One token, us, two / three an SM: N = 128,
@@ -134,11 +133,13 @@ int launch_short_t(const crc_problem& p, const uint16_t* hidden, const uint16_t*
 
 template <int NH, int V, bool ALL_VALID>
 int launch_short_for_n(const crc_problem& p, const uint16_t* hidden, const uint16_t* w_cat, int T,
-                       void* state, const crc_trace* trace, cudaStream_t stream) {
+                       void* state, const crc_trace* trace, bool persistent,
+                       cudaStream_t stream) {
     return trace_wanted(trace)
-               ? launch_short_t<NH, V, ALL_VALID, true>(p, hidden, w_cat, T, state, trace, stream)
+               ? launch_short_t<NH, V, ALL_VALID, true>(p, hidden, w_cat, T, state, trace,
+                                                        persistent, stream)
                : launch_short_t<NH, V, ALL_VALID, false>(p, hidden, w_cat, T, state, nullptr,
-                                                         stream);
+                                                         persistent, stream);
 }
 
 }  // namespace crc

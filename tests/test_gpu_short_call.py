@@ -86,6 +86,28 @@ def test_short_calls_of_many_clusters(C, name, traced):
     run_short_calls(C, THREE[name], traced, True)
 
 
+@pytest.mark.parametrize("w", [S.QWEN3_30B.with_(L=55, B=130, T=2, d=4104),
+                               S.QWEN3_30B.with_(L=48, B=200, T=4, d=72)], ids=["two", "four"])
+def test_a_small_workspace_keeps_short_calls(C, w):
+    """Calls that the persistent kernel takes when its workspace is there run as
+    short calls, not as the router's and the scan's launches, when it is not."""
+    p = C.problem_of(w)
+    W = C.synth_weights(w.L, w.N, w.d, seed=3)
+    h, _ = C.synth_hidden(w.B, w.T, w.L, w.d, seed=4)
+    got = []
+    for nbytes, short in ((C.crc_workspace_bytes(p, 1), 1), (C.crc_fused_workspace_bytes(p), 0)):
+        ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        st = C.State(p)
+        C.crc_profile_begin()
+        C.route_and_cache(p, h, W, st, None, workspace=ws)
+        kt = C.crc_profile_end()
+        assert kt["fused"]["launches"] == 1 and kt["short"]["launches"] == short
+        got.append(st.read(want_caches=True, want_retention=True, want_chain_counters=True))
+    for name in ("cache_bits", "chain_counters"):
+        assert (got[0][name] == got[1][name]).all(), name
+    assert (got[0]["retention"].view("u4") == got[1]["retention"].view("u4")).all()
+
+
 def test_one_state_over_short_and_persistent_calls(C):
     """A serving loop's mix on one state: single tokens, chunks and long calls in
     turn, traced and not, against one scan of the same scores in the same pieces."""
