@@ -20,13 +20,13 @@
 //
 // What bounds the step: the integer pipe (16 lanes a scheduler) when many
 // chains share an SM, and for a few chains the latency of some 300 dependent
-// instructions, a max/min redux.sync taking 23 cycles, an add 48.  Against the
-// step with integer masks, selects and one reduction after another: Qwen3
-// shape, stand-alone scan of 64 streams x 1000 tokens, 1.62 -> 1.27 ms for the
-// method, 1.06 -> 0.85 LRU, 1.24 -> 0.91 LFU, 1.39 -> 1.31 LRFU, 1.57 -> 1.39
-// Spatio-only; GPT-OSS shape (one expert a lane) 0.64 -> 0.44 ms, 0.34 -> 0.32,
-// 0.36 -> 0.33, 0.43 -> 0.43, 0.63 -> 0.52; one stream through the fused
-// kernel, 0.82 -> 0.65 us a token.
+// instructions, a max/min redux.sync taking 23 cycles, an add 48.  So residency
+// is held in floats and worked on by the FMA pipe.  Integer masks and selects
+// with one reduction after another / this form, ms: Qwen3 shape, stand-alone scan
+// of 64 streams x 1000 tokens, method 1.62 / 1.27, LRU 1.06 / 0.85, LFU 1.24 /
+// 0.91, LRFU 1.39 / 1.31, Spatio-only 1.57 / 1.39; GPT-OSS shape (one expert a
+// lane) 0.64 / 0.44, 0.34 / 0.32, 0.36 / 0.33, 0.43 / 0.43, 0.63 / 0.52; one
+// stream through the fused kernel, 0.82 / 0.65 us a token.
 #pragma once
 
 #include "crc_device.cuh"
@@ -1052,8 +1052,12 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
         // token t + j for t a multiple of 32; th is the current token's.  A
         // rank-order trace takes the whole order instead and needs none (one
         // token, N = 128, K = 32, 64 streams x 24 layers: 24.6 us with the
-        // thresholds, 9.5 without).
+        // thresholds, 9.5 without).  They are taken within the step, or before it
+        // for the widest network, whose registers weigh on it (us, before / within:
+        // K = 8, 40 streams x 600 tokens, Qwen3 shape, 598 / 588; N = 128, 64 streams
+        // x 24 layers x 300, K = 16 320 / 307, K = 32 405 / 451).
         float theta = 0.f, th = 0.f;
+        constexpr bool BEFORE = KP > 16;
         auto thresholds = [&](int t) {
             if (t + lane < T && unit_ok(t + lane, l))
                 theta = row_theta_k<KP>(row0 + (size_t)(t + lane) * tok, N, a.K);
@@ -1065,6 +1069,7 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
             ring_read<V>(&from[0][lane * V], pR);
             ring_read<V>(&from[1][lane * V], pT);
             ring_read<V>(&from[2][lane * V], pS);
+            if (!BEFORE && !rank_order && (t & 31) == 0) thresholds(t);
             Sel<V> s;
             float sT[V];
             if (!rank_order) sel_above<V, ALL_VALID>(pR, th, valid, s);
@@ -1104,7 +1109,7 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
 #pragma unroll 1
         for (int t = 0; t < T; ++t) {
             load(t + D - 1);
-            if (!rank_order && (t & 31) == 0) thresholds(t);   // its loads overlap the copies
+            if (BEFORE && !rank_order && (t & 31) == 0) thresholds(t);
             ring_wait<D - 1>();                  // token t's copies have landed
             step(t);
             th = __shfl_sync(kFull, theta, (t + 1) & 31);

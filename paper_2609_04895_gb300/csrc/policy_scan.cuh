@@ -232,8 +232,14 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
             ring_commit();
             up += tok;
         };
-        float theta = 0.f, th = 0.f;             // Top-K thresholds: lane j token t + j's; t's
-        auto thresholds = [&](int t) {           // (a rank-order trace needs none)
+        // Top-K thresholds: lane j token t + j's; t's.  (A rank-order trace needs none.)
+        // Taken within the step, or before it for Spatio-only, whose step holds more,
+        // and for the widest network (40 streams x 600 tokens, Qwen3 shape, us,
+        // before / within: LRU 385 / 380, LFU 412 / 404, LRFU 594 / 586, Spatio-only
+        // 617 / 627; LFU, K = 32, 64 streams x 24 layers x 300 331 / 352).
+        float theta = 0.f, th = 0.f;
+        constexpr bool BEFORE = POL == CRC_POLICY_SPATIO_LRU || KP > 16;
+        auto thresholds = [&](int t) {
             if (t + lane < T) theta = row_theta_k<KP>(row0 + (size_t)(t + lane) * tok, N, a.K);
             th = __shfl_sync(kFull, theta, 0);
         };
@@ -241,6 +247,7 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
             float pR[V], pS[V];
             ring_read<V>(&mine[t % D][0][lane * V], pR);
             ring_read<V>(&mine[t % D][ROWS - 1][lane * V], pS);
+            if (!BEFORE && !rank_order && (t & 31) == 0) thresholds(t);
             Sel<V> s;
             const size_t unit = ((size_t)b * a.trace_T + a.trace_t0 + t) * L + l;
             if (rank_order)
@@ -259,7 +266,7 @@ __global__ void __launch_bounds__(32 * kScanWarps, (V >= 8 ? 12 : 24) / kScanWar
 #pragma unroll 1
         for (int t = 0; t < T; ++t) {
             load(t + D - 1);
-            if (!rank_order && (t & 31) == 0) thresholds(t);
+            if (BEFORE && !rank_order && (t & 31) == 0) thresholds(t);
             ring_wait<D - 1>();                  // token t's copies have landed
             step(t);
             th = __shfl_sync(kFull, theta, (t + 1) & 31);
