@@ -814,7 +814,9 @@ def rooflines(kt, w, heads, steps, ms, ms_per_step, scan_heads=None, clocks=None
     elif dom == "router":
         flops = 2.0 * w.d * heads * w.N * w.units * steps
         bytes_ = (2.0 * w.d + 4.0 * heads * w.N) * w.units * steps   # + scores written
-        kname = f"router_heads_kernel<{w.N},{heads}>"
+        # N = 128: router_pair_kernel or router_heads_kernel, by the call's rounds of tiles
+        kname = ("router_pair_kernel / " if w.N == 128 else "") + \
+            f"router_heads_kernel<{w.N},{heads}>"
     else:
         flops, bytes_ = algorithmic(w, w.units, heads)
         flops, bytes_ = flops * steps, bytes_ * steps

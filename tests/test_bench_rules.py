@@ -101,6 +101,17 @@ def test_one_token_steps_are_named_by_their_own_kernel(monkeypatch):
     assert bench.source_hash(roof["kernel"]) != bench.source_hash("fused_route_cache_kernel<128,3>")
 
 
+def test_router_heads_are_named_by_both_kernels(monkeypatch):
+    """Heads of 128 experts run on CTA pairs or on single CTAs; the line says so."""
+    monkeypatch.setattr(bench, "peaks", lambda: (dict(PK), "measured"))
+    kt = {"fused": {"ms": 0.0, "launches": 0}, "router": {"ms": 3.6, "launches": 1},
+          "scan": {"ms": 0.0, "launches": 0}}
+    for w, name in ((S.QWEN3_30B, "router_pair_kernel / router_heads_kernel<128,3>"),
+                    (S.GPT_OSS_20B, "router_heads_kernel<32,3>")):
+        roof, _, _ = bench.rooflines(kt, w, 3, 1, 3.6, 3.6)
+        assert roof["kernel"] == name and bench.kernel_family(name) == "router"
+
+
 def test_every_kernel_source_belongs_to_a_family():
     """The files that define the profiled kernels are among their families' sources."""
     csrc = os.path.join(ROOT, "paper_2609_04895_gb300", "csrc")
