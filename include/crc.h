@@ -236,19 +236,20 @@ size_t crc_fused_workspace_bytes(const crc_problem *p);
  * hidden_dev bf16 [B][T][L][d]; w_cat_dev bf16 [L][3N][d] (the S head is
  * not computed when R = 0).  The router scores never leave the workspace.
  * With K <= 8 and a trace that leaves topk_dev NULL (or no trace), short calls
- * (one or two tokens, up to 64 when few enough) run as one kernel that uses no
- * workspace, and with workspace_bytes >= crc_fused_workspace_bytes(p) the others
- * as one persistent fused kernel; for N = 128 with an even number of tiles a
- * layer its GEMM runs on CTA pairs (clusters of two, tcgen05 cta_group::2),
- * otherwise one CTA per tile.  All give the same
- * results.  The pair kernel is a cooperative cluster launch; with the
- * environment variable CRC_PLAIN_CLUSTER_LAUNCH=1 (read once per process) it
- * is launched without the cooperative attribute, for kernel profilers that
- * cannot replay cooperative cluster launches (same kernel, same grid, which
- * fits the GPU at once; a stall would end in CRC_ETIMEOUT).  Without that
- * workspace, workspace_dev holds the scores of one chunk of tokens, the chunk length being the largest that fits (at least one
- * token must fit, see crc_workspace_bytes).  256-byte alignment for the
- * workspace. */
+ * (one token, two unless the rows are wide and many, up to 64 when few enough)
+ * run as one kernel that uses no workspace, and with workspace_bytes >=
+ * crc_fused_workspace_bytes(p) the others as one persistent fused kernel; for
+ * N = 128 with an even number of stream groups (tiles of a layer and token
+ * block) its GEMM runs on CTA pairs (clusters of two, tcgen05 cta_group::2),
+ * otherwise one CTA per tile.  All give the same results.  The pair kernel is
+ * a cooperative cluster launch; with the environment variable
+ * CRC_PLAIN_CLUSTER_LAUNCH=1 (read once per process) it is launched without
+ * the cooperative attribute, for kernel profilers that cannot replay
+ * cooperative cluster launches (same kernel, same grid, which fits the GPU at
+ * once; a stall would end in CRC_ETIMEOUT).  Without that workspace,
+ * workspace_dev holds the scores of one chunk of tokens, the chunk length being
+ * the largest that fits (at least one token must fit, see
+ * crc_workspace_bytes).  256-byte alignment for the workspace. */
 int crc_route_and_cache(const crc_problem *p, const uint16_t *hidden_dev,
                         const uint16_t *w_cat_dev, int32_t T, void *state_dev,
                         size_t state_bytes, const crc_trace *trace,

@@ -524,8 +524,8 @@ __global__ void __launch_bounds__(512, 1)
     const int lane = threadIdx.x & 31;
     // PAIR: rank 0 issues the MMAs for both CTAs; the tile loops below step by
     // gridDim.x from blockIdx.x, so the two CTAs of a pair hold the adjacent
-    // tiles 2j and 2j + 1 (same token block and layer: the launch makes the
-    // stream count even) at every iteration.
+    // tiles 2j and 2j + 1 (same token block and layer: the launch takes pairs
+    // only for an even number of stream groups) at every iteration.
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
     const bool leader = rank == 0u;
 
@@ -583,11 +583,12 @@ __global__ void __launch_bounds__(512, 1)
                 const int rem = k % a.tiles_per_tb;
                 const int l = rem / a.n_bg, bg = rem % a.n_bg;
                 // The abort flag is asked for once a tile and looked at when the
-                // tile's loads are out.  Read before every K block, as it was, it
-                // put a trip to L2 between any two loads, a longer one with the
-                // item counter's atomics on the same line: N = 32, 64 x 1000
-                // tokens 1.90 ms, now 1.54; N = 128, 64 x 1024 4.07 -> 3.86,
-                // R = 0 48 x 777 1.96 -> 1.64.
+                // tile's loads are out: a read before every K block puts a trip to
+                // L2 between any two loads, a longer one with the item counter's
+                // atomics on the same line (every K block / once a tile, ms: N = 32,
+                // 64 x 1000 tokens 1.90 / 1.54; N = 128, 64 x 1024 4.07 / 3.86;
+                // R = 0, 48 x 777 1.96 / 1.64).  A stage that another role's abort
+                // leaves unfreed is waited for to the limit, as the MMA issuer waits.
                 const uint32_t aborted = ld_relaxed_u32(abort_flag);
                 for (int kb = 0; kb < a.kblocks; ++kb) {
                     const bool freed = PAIR ? mbar_wait_cluster(&empty_bar[stage], phase ^ 1)

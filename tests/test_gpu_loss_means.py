@@ -4,7 +4,7 @@ tokens are one task each.
 
 Both sides add the same fp32 losses in fp64, n = B (T - 1) L of them in some
 order: each sum is within n 2^-53 of the exact one (all terms >= 0), so they
-differ by at most 2 n 2^-53 of it, 1.4e-12 for the largest n here.
+differ by at most 2 n 2^-53 of it, 2.7e-12 for the largest n here.
 """
 import pytest
 
