@@ -4,7 +4,7 @@ In it every index a kernel derives -- stream, layer, chain, token, ring slot,
 tile row, the experts a step makes resident -- is checked against the bound
 of the array it addresses before use; a failed check latches CRC_EDEVICE and
 skips the access instead of touching memory (the stand-in for a memory
-checker, which this pool does not offer).  Slices of every configuration run
+checker where none can be run).  Slices of every configuration run
 on it -- the short-call kernel in both its launch forms, the persistent fused
 kernel with long and short token blocks on CTA pairs and on single CTAs, each
 with and without its trace, the chunked two-kernel path, the router heads on
